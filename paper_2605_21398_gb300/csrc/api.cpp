@@ -48,8 +48,10 @@ struct RefBufs {
     size_t cands_n = 0;
     RefineDev *dev = nullptr;   // per-request refinement tables of a launch
     size_t dev_n = 0;
-    int32_t *hint = nullptr;    // per-query witness triangle of the previous evaluation
+    int2 *hint = nullptr;       // per-query witness of the previous evaluation (leaf slot, packed barycentric point)
     size_t hint_n = 0;
+    int32_t *redo = nullptr;    // partials evaluated again in the order of a shared walk
+    size_t redo_n = 0;
     int32_t *grp = nullptr;     // candidate -> request
     size_t grp_n = 0;
     double *lb = nullptr;       // L-BFGS-B state per candidate (LB_ST doubles)
@@ -67,6 +69,7 @@ static void free_refbufs(RefBufs &b)
     cudaFree(b.dev);
     cudaFree(b.grp);
     cudaFree(b.hint);
+    cudaFree(b.redo);
     cudaFree(b.lb);
     cudaFree(b.active);
     b = RefBufs();
@@ -154,11 +157,8 @@ struct dock_object {
     double *o_dev = nullptr;
     // mesh for the refinement
     int64_t nv = 0, nt = 0;
-    float *Vf = nullptr;
-    int32_t *T = nullptr;
-    float *tri_sphere = nullptr;
-    int32_t *tri_order = nullptr;
-    BvhNode *nodes = nullptr;
+    LeafRec *leaf = nullptr;   // triangles in BVH leaf order
+    NodeRec *nodes = nullptr;
     int n_nodes = 0;
     size_t bytes = 0;
 };
@@ -798,7 +798,8 @@ static void build_bvh(const double *V, const int32_t *T, int64_t nt, std::vector
         nodes.push_back(BvhNode());
         nodes[it.node].left = l;
         nodes[it.node].right = r;
-        nodes[it.node].count = 0;
+        nodes[it.node].count = n;
+        nodes[it.node].pad = it.lo;
         stack.push_back({r, mid, it.hi});
         stack.push_back({l, it.lo, mid});
     }
@@ -858,13 +859,22 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     build_bins3(verts, tris, T, ob->o, cs, d3, cut, s3, i3);
     build_bins2(verts, tris, T, ob->o, cs, d2, s2, i2);
     // device buffers
-    double *dV = nullptr, *dcen = nullptr;
+    double *dV = nullptr;
+    float *dVf = nullptr, *dsph = nullptr;
+    int32_t *dorder = nullptr;
+    BvhNode *dnodes = nullptr;
+    size_t n_dnodes = 0;
     int32_t *dT = nullptr, *ds3 = nullptr, *di3 = nullptr, *ds2 = nullptr, *di2 = nullptr;
     uint8_t *dtouch = nullptr;
     double2 *w1 = nullptr, *w2 = nullptr;
     size_t tmp_bytes = 0;
     auto cleanup_tmp = [&]() {
         dfree(ctx, dV, sizeof(double) * 3 * V);
+        dfree(ctx, dVf, sizeof(float) * 3 * V);
+        dfree(ctx, dsph, sizeof(float) * 4 * T);
+        dfree(ctx, dorder, sizeof(int32_t) * T);
+        dfree(ctx, dnodes, sizeof(BvhNode) * n_dnodes);
+        dfree(ctx, dT, sizeof(int32_t) * 3 * T);
         dfree(ctx, ds3, sizeof(int32_t) * s3.size());
         dfree(ctx, di3, sizeof(int32_t) * i3.size());
         dfree(ctx, ds2, sizeof(int32_t) * s2.size());
@@ -872,7 +882,6 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
         dfree(ctx, dtouch, (size_t)T);
         dfree(ctx, w1, sizeof(double2) * (size_t)N * N * (N + 1));
         dfree(ctx, w2, sizeof(double2) * (size_t)N * M * (N + 1));
-        (void)dcen;
     };
     auto bail = [&](dock_status st) {
         cleanup_tmp();
@@ -880,8 +889,7 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
         return st;
     };
     if ((s = dalloc(ctx, (void **)&dV, sizeof(double) * 3 * V, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&dT, sizeof(int32_t) * 3 * T, &ob->bytes)) != DOCK_OK) return bail(s);
-    ob->T = dT;
+    if ((s = dalloc(ctx, (void **)&dT, sizeof(int32_t) * 3 * T, &tmp_bytes)) != DOCK_OK) return bail(s);
     if ((s = dalloc(ctx, (void **)&ds3, sizeof(int32_t) * s3.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
     if ((s = dalloc(ctx, (void **)&di3, sizeof(int32_t) * i3.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
     if ((s = dalloc(ctx, (void **)&ds2, sizeof(int32_t) * s2.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
@@ -936,14 +944,19 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     ob->nv = V;
     ob->nt = T;
     ob->n_nodes = (int)nodes.size();
-    if ((s = dalloc(ctx, (void **)&ob->Vf, sizeof(float) * 3 * V, &ob->bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->tri_sphere, sizeof(float) * 4 * T, &ob->bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->tri_order, sizeof(int32_t) * T, &ob->bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->nodes, sizeof(BvhNode) * nodes.size(), &ob->bytes)) != DOCK_OK) return bail(s);
-    CKB(cudaMemcpyAsync(ob->Vf, vf.data(), sizeof(float) * 3 * V, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(ob->tri_sphere, tsph.data(), sizeof(float) * 4 * T, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(ob->tri_order, order.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(ob->nodes, nodes.data(), sizeof(BvhNode) * nodes.size(), cudaMemcpyHostToDevice, st));
+    if ((s = dalloc(ctx, (void **)&dVf, sizeof(float) * 3 * V, &tmp_bytes)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&dsph, sizeof(float) * 4 * T, &tmp_bytes)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&dorder, sizeof(int32_t) * T, &tmp_bytes)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&ob->leaf, leaf_bytes() * T, &ob->bytes)) != DOCK_OK) return bail(s);
+    n_dnodes = nodes.size();
+    if ((s = dalloc(ctx, (void **)&dnodes, sizeof(BvhNode) * n_dnodes, &tmp_bytes)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&ob->nodes, node_bytes() * n_dnodes, &ob->bytes)) != DOCK_OK) return bail(s);
+    CKB(cudaMemcpyAsync(dVf, vf.data(), sizeof(float) * 3 * V, cudaMemcpyHostToDevice, st));
+    CKB(cudaMemcpyAsync(dsph, tsph.data(), sizeof(float) * 4 * T, cudaMemcpyHostToDevice, st));
+    CKB(cudaMemcpyAsync(dorder, order.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
+    CKB(cudaMemcpyAsync(dnodes, nodes.data(), sizeof(BvhNode) * nodes.size(), cudaMemcpyHostToDevice, st));
+    CKB(launch_leaf_records((int)T, dVf, dT, dsph, dorder, ob->leaf, st));
+    CKB(launch_node_records((int)n_dnodes, dnodes, ob->leaf, ob->nodes, st));
     int herr = 0;
     CKB(cudaMemcpyAsync(&herr, ctx->errflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     CKB(cudaStreamSynchronize(st));
@@ -970,10 +983,7 @@ extern "C" void dock_object_free(dock_object *ob)
     cudaFree(ob->spec_pen);
     cudaFree(ob->cells);
     cudaFree(ob->o_dev);
-    cudaFree(ob->Vf);
-    cudaFree(ob->T);
-    cudaFree(ob->tri_sphere);
-    cudaFree(ob->tri_order);
+    cudaFree(ob->leaf);
     cudaFree(ob->nodes);
     ctx->held = ctx->held >= ob->bytes ? ctx->held - ob->bytes : 0;
     delete ob;
@@ -2163,10 +2173,7 @@ extern "C" dock_status dock_sample_so3(const dock_search_desc *d, double *quats)
 static RefineDev make_refine_dev(const dock_object *ob, const dock_sweep *sw, const dock_params *p)
 {
     RefineDev D;
-    D.Vf = ob->Vf;
-    D.T = ob->T;
-    D.tri_sphere = ob->tri_sphere;
-    D.tri_order = ob->tri_order;
+    D.leaf = ob->leaf;
     D.nodes = ob->nodes;
     D.poses = sw->poses;
     D.P = (int)sw->P;
@@ -2191,6 +2198,7 @@ static dock_status ref_buffers(dock_ctx *ctx, RefBufs &rb, int K, int nblk)
     if ((s = ensure(ctx, (void **)&rb.state, &rb.state_n, (size_t)K * REF_ST, sizeof(double))) != DOCK_OK) return s;
     if ((s = ensure(ctx, (void **)&rb.acc, &rb.acc_n, (size_t)K * nblk * REF_NACC, sizeof(double))) != DOCK_OK) return s;
     if ((s = ensure(ctx, (void **)&rb.prm, &rb.prm_n, 16, sizeof(double))) != DOCK_OK) return s;
+    if ((s = ensure(ctx, (void **)&rb.redo, &rb.redo_n, (size_t)K * nblk + 1, sizeof(int32_t))) != DOCK_OK) return s;
     if ((s = ensure(ctx, (void **)&rb.cands, &rb.cands_n, (size_t)K, cand_bytes())) != DOCK_OK) return s;
     return DOCK_OK;
 }
@@ -2281,8 +2289,8 @@ static dock_status refine_loop(dock_ctx *ctx, RefBufs &rb, int K, int nblk, int 
     CK(ctx, cudaMemcpyAsync(rb.prm, prm, sizeof(prm), cudaMemcpyHostToDevice, st));
     CandF *cf = (CandF *)rb.cands;
     dock_status s;
-    if ((s = ensure(ctx, (void **)&rb.hint, &rb.hint_n, (size_t)K * nblk * 128, sizeof(int32_t))) != DOCK_OK) return s;
-    CK(ctx, cudaMemsetAsync(rb.hint, 0xFF, sizeof(int32_t) * (size_t)K * nblk * 128, st));   // -1: no hint yet
+    if ((s = ensure(ctx, (void **)&rb.hint, &rb.hint_n, (size_t)K * nblk * 128, sizeof(int2))) != DOCK_OK) return s;
+    CK(ctx, cudaMemsetAsync(rb.hint, 0xFF, sizeof(int2) * (size_t)K * nblk * 128, st));   // -1: no hint yet
     if (p->solver == DOCK_SOLVER_LBFGSB) {
         // L-BFGS-B (Sec. V-C as printed): rounds of one evaluation (J and
         // grad J at every active candidate's trial twist) and one solver
@@ -2293,7 +2301,7 @@ static dock_status refine_loop(dock_ctx *ctx, RefBufs &rb, int K, int nblk, int 
         for (int r = 0; r < p->lbfgs_evals; ++r) {
             {
                 Prof pr(ctx, "refine_eval", st);
-                CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk, cf, rb.acc, true, nullptr, nullptr, nullptr, st,
+                CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk * REF_WARPS, cf, rb.acc, true, nullptr, nullptr, nullptr, rb.redo, st,
                                            rb.hint, rb.active));
             }
             Prof pr(ctx, "refine_lbfgs", st);
@@ -2306,7 +2314,7 @@ static dock_status refine_loop(dock_ctx *ctx, RefBufs &rb, int K, int nblk, int 
     for (int it = 0; it < iters; ++it) {
         {
             Prof pr(ctx, "refine_eval", st);
-            CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk, cf, rb.acc, true, nullptr, nullptr, nullptr, st,
+            CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk * REF_WARPS, cf, rb.acc, true, nullptr, nullptr, nullptr, rb.redo, st,
                                        rb.hint));
         }
         Prof pr(ctx, "refine_solve", st);
@@ -2314,7 +2322,7 @@ static dock_status refine_loop(dock_ctx *ctx, RefBufs &rb, int K, int nblk, int 
     }
     {
         Prof pr(ctx, "refine_eval", st);
-        CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk, cf, rb.acc, false, nullptr, nullptr, nullptr, st,
+        CK(ctx, launch_refine_eval(rb.dev, rb.grp, K, nblk * REF_WARPS, cf, rb.acc, false, nullptr, nullptr, nullptr, rb.redo, st,
                                    rb.hint));
     }
     CK(ctx, launch_refine_solve(K, nblk * REF_WARPS, rb.state, rb.acc, rb.prm, 2, cf, st));
@@ -2471,8 +2479,8 @@ static dock_status objective_impl(dock_ctx *ctx, const dock_object *ob, const do
     CK(ctx, launch_refine_solve(B, nblk * REF_WARPS, ctx->ref.state, ctx->ref.acc, ctx->ref.prm, 0, cf, st));
     {
         Prof pr(ctx, grad ? "objective_adjoint" : "objective_fwd");
-        CK(ctx, launch_refine_eval(ctx->ref.dev, nullptr, B, nblk, cf, ctx->ref.acc, grad != nullptr, nullptr, nullptr,
-                                   nullptr, st));
+        CK(ctx, launch_refine_eval(ctx->ref.dev, nullptr, B, nblk * REF_WARPS, cf, ctx->ref.acc, grad != nullptr, nullptr, nullptr,
+                                   nullptr, ctx->ref.redo, st));
     }
     CK(ctx, launch_finish_objective(B, nblk * REF_WARPS, ctx->ref.state, ctx->ref.acc, p->lambda, J, grad, gJ, st));
     return DOCK_OK;
@@ -2531,7 +2539,7 @@ extern "C" dock_status dock_distances(dock_ctx *ctx, const dock_object *ob, cons
     cudaError_t e = cudaMemcpyAsync(ctx->ref.state, stv.data(), sizeof(double) * stv.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = launch_refine_solve(B, nblk * REF_WARPS, ctx->ref.state, ctx->ref.acc, ctx->ref.prm, 0, cf, st);
     if (e == cudaSuccess)
-        e = launch_refine_eval(ctx->ref.dev, nullptr, B, nblk, cf, ctx->ref.acc, false, buf, buf + n, buf + 4 * n, st);
+        e = launch_refine_eval(ctx->ref.dev, nullptr, B, nblk * REF_WARPS, cf, ctx->ref.acc, false, buf, buf + n, buf + 4 * n, ctx->ref.redo, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d, buf, sizeof(float) * n, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(witness, buf + n, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(normal, buf + 4 * n, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, st);

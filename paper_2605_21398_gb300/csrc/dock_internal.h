@@ -169,16 +169,20 @@ struct BvhNode {
     float c[3];    // sphere centre (object frame)
     float rad;     // sphere radius
     int32_t left;  // child index, or -1 for a leaf
-    int32_t right; // right child, or the leaf's first slot in the triangle order
-    int32_t count; // leaf triangle count
-    int32_t pad;
+    int32_t right; // right child (left + 1), or the leaf's first slot in the triangle order
+    int32_t count; // triangles below the node
+    int32_t pad;   // interior node: first slot of its triangles
 };
+struct LeafRec;               // one triangle of a leaf (k_refine.cu)
+struct NodeRec;               // one BVH node (k_refine.cu)
+size_t leaf_bytes();
+size_t node_bytes();
+cudaError_t launch_node_records(int n, const BvhNode *in, const LeafRec *leaf, NodeRec *out, cudaStream_t st);
+cudaError_t launch_leaf_records(int n, const float *Vf, const int32_t *T, const float *tri_sphere,
+                                const int32_t *tri_order, LeafRec *out, cudaStream_t st);
 struct RefineDev {
-    const float *Vf;          // V x 3
-    const int32_t *T;         // T x 3
-    const float *tri_sphere;  // T x 4 (centre, radius), object frame
-    const int32_t *tri_order; // leaf slot -> triangle index
-    const BvhNode *nodes;
+    const LeafRec *leaf;      // triangles in leaf order
+    const NodeRec *nodes;
     const PoseRec *poses;
     int P;
     float r, L;
@@ -190,22 +194,25 @@ struct CandF;                 // per-candidate FP32 pose data (k_refine.cu)
 size_t cand_bytes();
 constexpr int REF_ST = 24;    // doubles of refinement state per candidate
 constexpr int REF_NACC = 28;  // accumulated J, grad (6), Gauss-Newton upper triangle (21)
-constexpr int REF_WARPS = 4;  // warps per block of the refinement evaluation (one partial sum each)
-// hints (optional, K x nblk x 128): each query's witness triangle, read as a
-// starting bound and overwritten; -1 = none.
+constexpr int REF_WARPS = 4;  // partial sums (32 poses each) per 128 poses of the refinement evaluation
+// nwarp: partial sums per candidate (one per 32 poses), a multiple of REF_WARPS.
+// hints (optional, K x nwarp x 32): each query's witness (leaf slot, packed
+// barycentric point), read as a starting bound and overwritten; slot -1 = none.
 // active (optional, K): candidates whose flag is 0 are skipped.
-cudaError_t launch_refine_eval(const RefineDev *Dt, const int32_t *grp, int K, int nblk, const CandF *cands,
+// redo (K nwarp + 1 entries): list of the partials evaluated a second time.
+cudaError_t launch_refine_eval(const RefineDev *Dt, const int32_t *grp, int K, int nwarp, const CandF *cands,
                                double *acc_part, bool grad, float *dist_out, float *wit_out, float *nrm_out,
-                               cudaStream_t st, int32_t *hints = nullptr, const int32_t *active = nullptr);
+                               int32_t *redo, cudaStream_t st, int2 *hints = nullptr,
+                               const int32_t *active = nullptr);
 // L-BFGS-B refinement (Sec. V-C): LB_ST doubles of solver state per candidate.
 constexpr int LB_M = 8;                  // stored (s, y) pairs
 constexpr int LB_ST = 32 + 13 * LB_M;
-cudaError_t launch_lbfgs(int K, int nblk, double *state, const double *acc_part, const double *prm, double *lbs,
+cudaError_t launch_lbfgs(int K, int nwarp, double *state, const double *acc_part, const double *prm, double *lbs,
                          int32_t *active, CandF *cands, int phase, cudaStream_t st);
-cudaError_t launch_refine_solve(int K, int nblk, double *state, const double *acc_part, const double *prm, int mode,
+cudaError_t launch_refine_solve(int K, int nwarp, double *state, const double *acc_part, const double *prm, int mode,
                                 CandF *cands, cudaStream_t st);
 cudaError_t launch_set_xi(int B, const float *xi, double *state, cudaStream_t st);
-cudaError_t launch_finish_objective(int B, int nblk, const double *state, const double *acc_part, double lam, float *J,
+cudaError_t launch_finish_objective(int B, int nwarp, const double *state, const double *acc_part, double lam, float *J,
                                     float *grad, const float *gJ, cudaStream_t st);
 
 // Search on library-owned scratch (k_noalloc.cu): limits of that scratch.
