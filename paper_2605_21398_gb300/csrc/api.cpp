@@ -647,162 +647,99 @@ static bool valid_N(int N) { return N == 32 || N == 64 || N == 96 || N == 128; }
 // ---------------------------------------------------------------------------
 // object
 // ---------------------------------------------------------------------------
-static void build_bins3(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
-                        double pad, std::vector<int32_t> &start, std::vector<int32_t> &items)
-{
-    int64_t nc = (int64_t)d[0] * d[1] * d[2];
-    std::vector<int32_t> cnt(nc + 1, 0);
-    for (int pass = 0; pass < 2; ++pass) {
-        if (pass == 1) {
-            start.assign(nc + 1, 0);
-            for (int64_t c = 0; c < nc; ++c) start[c + 1] = start[c] + cnt[c];
-            items.assign(start[nc] > 0 ? start[nc] : 1, 0);
-            std::fill(cnt.begin(), cnt.end(), 0);
-        }
-        for (int64_t t = 0; t < nt; ++t) {
-            int lo[3], hi[3];
-            bool ok = true;
-            for (int a = 0; a < 3; ++a) {
-                double x0 = V[3 * T[3 * t] + a], x1 = V[3 * T[3 * t + 1] + a], x2 = V[3 * T[3 * t + 2] + a];
-                double mn = std::min(x0, std::min(x1, x2)) - pad, mx = std::max(x0, std::max(x1, x2)) + pad;
-                lo[a] = std::max(0, (int)floor((mn - o[a]) / cs));
-                hi[a] = std::min(d[a] - 1, (int)floor((mx - o[a]) / cs));
-                if (lo[a] > hi[a]) ok = false;
-            }
-            if (!ok) continue;
-            for (int z = lo[2]; z <= hi[2]; ++z)
-                for (int y = lo[1]; y <= hi[1]; ++y)
-                    for (int x = lo[0]; x <= hi[0]; ++x) {
-                        int64_t c = ((int64_t)z * d[1] + y) * d[0] + x;
-                        if (pass == 0) cnt[c]++;
-                        else items[start[c] + cnt[c]++] = (int32_t)t;
-                    }
-        }
-    }
-}
+// The tree over triangles (object frame): median split on the longest centroid
+// axis, leaves of <= 4 triangles.  Node spheres and slabs are made on the device
+// (launch_node_records); the host decides the splits.  A node's centroids are
+// moved with its triangles, so every pass over them is sequential; subtrees of
+// many triangles are built by threads of their own (the number of nodes below n
+// triangles depends on n alone, so every subtree knows its place).
+struct BvhItem {
+    double c[3];   // centre of the triangle's box
+    int32_t t;
+};
 
-static void build_bins2(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
-                        std::vector<int32_t> &start, std::vector<int32_t> &items)
-{
-    int64_t nc = (int64_t)d[0] * d[1];
-    std::vector<int32_t> cnt(nc + 1, 0);
-    for (int pass = 0; pass < 2; ++pass) {
-        if (pass == 1) {
-            start.assign(nc + 1, 0);
-            for (int64_t c = 0; c < nc; ++c) start[c + 1] = start[c] + cnt[c];
-            items.assign(start[nc] > 0 ? start[nc] : 1, 0);
-            std::fill(cnt.begin(), cnt.end(), 0);
-        }
-        for (int64_t t = 0; t < nt; ++t) {
-            int lo[2], hi[2];
-            bool ok = true;
-            for (int k = 0; k < 2; ++k) {
-                int a = k + 1;
-                double x0 = V[3 * T[3 * t] + a], x1 = V[3 * T[3 * t + 1] + a], x2 = V[3 * T[3 * t + 2] + a];
-                double mn = std::min(x0, std::min(x1, x2)), mx = std::max(x0, std::max(x1, x2));
-                lo[k] = std::max(0, (int)floor((mn - o[a]) / cs));
-                hi[k] = std::min(d[k] - 1, (int)floor((mx - o[a]) / cs));
-                if (lo[k] > hi[k]) ok = false;
-            }
-            if (!ok) continue;
-            for (int z = lo[1]; z <= hi[1]; ++z)
-                for (int y = lo[0]; y <= hi[0]; ++y) {
-                    int64_t c = (int64_t)z * d[0] + y;
-                    if (pass == 0) cnt[c]++;
-                    else items[start[c] + cnt[c]++] = (int32_t)t;
-                }
-        }
-    }
-}
+struct BvhBuilder {
+    std::vector<BvhItem> items;
+    std::vector<BvhNode> nodes;
+    std::vector<int32_t> order;   // leaf slot -> triangle
+    static constexpr int THREAD_MIN = 4096;   // triangles that are worth a thread (about 1 ms)
 
-// BVH over triangles (object frame): median split on the longest centroid
-// axis, leaves of <= 4 triangles; node spheres enclose their triangles.
-static void build_bvh(const double *V, const int32_t *T, int64_t nt, std::vector<BvhNode> &nodes,
-                      std::vector<int32_t> &order, std::vector<float> &tri_sphere)
-{
-    order.resize(nt);
-    std::vector<double> cen(nt * 3);
-    tri_sphere.resize(nt * 4);
-    for (int64_t t = 0; t < nt; ++t) {
-        order[t] = (int32_t)t;
-        double lo[3], hi[3];
-        for (int a = 0; a < 3; ++a) {
-            double x0 = V[3 * T[3 * t] + a], x1 = V[3 * T[3 * t + 1] + a], x2 = V[3 * T[3 * t + 2] + a];
-            lo[a] = std::min(x0, std::min(x1, x2));
-            hi[a] = std::max(x0, std::max(x1, x2));
-            cen[3 * t + a] = 0.5 * (lo[a] + hi[a]);
+    // nodes of a tree over n triangles
+    static int64_t size(int64_t n)
+    {
+        // n / 2 and n - n / 2 differ by at most one: two sizes per level
+        int64_t a = n, ca = 1, cb = 0, total = 0;   // ca trees of a triangles, cb of a + 1
+        while (ca + cb > 0) {
+            total += ca + cb;
+            // halves of a and a + 1 that are split again
+            const int64_t h = a / 2;
+            int64_t nh = 0, nh1 = 0;
+            if (a > 4) { if (a & 1) { nh += ca; nh1 += ca; } else nh += 2 * ca; }
+            if (a + 1 > 4) { if ((a + 1) & 1) { nh += cb; nh1 += cb; } else nh1 += 2 * cb; }
+            a = h;
+            ca = nh;
+            cb = nh1;
         }
-        double rad = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            const double *v = V + 3 * T[3 * t + k];
-            double dx = v[0] - cen[3 * t], dy = v[1] - cen[3 * t + 1], dz = v[2] - cen[3 * t + 2];
-            rad = std::max(rad, sqrt(dx * dx + dy * dy + dz * dz));
-        }
-        for (int a = 0; a < 3; ++a) tri_sphere[4 * t + a] = (float)cen[3 * t + a];
-        tri_sphere[4 * t + 3] = (float)(rad * (1.0 + 1e-6) + 1e-6);
+        return total;
     }
-    nodes.clear();
-    nodes.reserve(2 * nt / 2 + 8);
-    struct Item { int node, lo, hi; };
-    std::vector<Item> stack;
-    nodes.push_back(BvhNode());
-    stack.push_back({0, 0, (int)nt});
-    while (!stack.empty()) {
-        Item it = stack.back();
-        stack.pop_back();
-        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-        for (int i = it.lo; i < it.hi; ++i) {
-            int t = order[i];
-            for (int k = 0; k < 3; ++k) {
-                const double *v = V + 3 * T[3 * t + k];
-                for (int a = 0; a < 3; ++a) { lo[a] = std::min(lo[a], v[a]); hi[a] = std::max(hi[a], v[a]); }
-            }
-        }
-        double c[3] = {0.5 * (lo[0] + hi[0]), 0.5 * (lo[1] + hi[1]), 0.5 * (lo[2] + hi[2])};
-        double rad = 0.0;
-        for (int i = it.lo; i < it.hi; ++i) {
-            int t = order[i];
-            for (int k = 0; k < 3; ++k) {
-                const double *v = V + 3 * T[3 * t + k];
-                double dx = v[0] - c[0], dy = v[1] - c[1], dz = v[2] - c[2];
-                rad = std::max(rad, sqrt(dx * dx + dy * dy + dz * dz));
-            }
-        }
-        BvhNode &nd = nodes[it.node];
-        for (int a = 0; a < 3; ++a) nd.c[a] = (float)c[a];
-        nd.rad = (float)(rad * (1.0 + 1e-6) + 1e-6);
+
+    // node over items [lo, hi); its descendants take nodes [next, ...)
+    void build(int node, int lo, int hi, int64_t next)
+    {
+        const int n = hi - lo;
+        BvhNode &nd = nodes[node];
+        nd.first = lo;
+        nd.count = n;
         nd.pad = 0;
-        int n = it.hi - it.lo;
         if (n <= 4) {
             nd.left = -1;
-            nd.right = it.lo;
-            nd.count = n;
-            continue;
+            for (int i = lo; i < hi; ++i) order[i] = items[i].t;
+            return;
         }
+        double clo[3] = {1e300, 1e300, 1e300}, chi[3] = {-1e300, -1e300, -1e300};
+        for (int i = lo; i < hi; ++i)
+            for (int a = 0; a < 3; ++a) {
+                clo[a] = std::min(clo[a], items[i].c[a]);
+                chi[a] = std::max(chi[a], items[i].c[a]);
+            }
         int ax = 0;
         double ext = -1;
-        double clo[3] = {1e300, 1e300, 1e300}, chi[3] = {-1e300, -1e300, -1e300};
-        for (int i = it.lo; i < it.hi; ++i)
-            for (int a = 0; a < 3; ++a) {
-                clo[a] = std::min(clo[a], cen[3 * order[i] + a]);
-                chi[a] = std::max(chi[a], cen[3 * order[i] + a]);
-            }
         for (int a = 0; a < 3; ++a) if (chi[a] - clo[a] > ext) { ext = chi[a] - clo[a]; ax = a; }
-        int mid = (it.lo + it.hi) / 2;
-        std::nth_element(order.begin() + it.lo, order.begin() + mid, order.begin() + it.hi,
-                         [&](int a, int b) { return cen[3 * a + ax] < cen[3 * b + ax] ||
-                                                   (cen[3 * a + ax] == cen[3 * b + ax] && a < b); });
-        int l = (int)nodes.size();
-        nodes.push_back(BvhNode());
-        int r = (int)nodes.size();
-        nodes.push_back(BvhNode());
-        nodes[it.node].left = l;
-        nodes[it.node].right = r;
-        nodes[it.node].count = n;
-        nodes[it.node].pad = it.lo;
-        stack.push_back({r, mid, it.hi});
-        stack.push_back({l, it.lo, mid});
+        const int mid = (int)(((int64_t)lo + hi) / 2);
+        std::nth_element(items.begin() + lo, items.begin() + mid, items.begin() + hi,
+                         [ax](const BvhItem &x, const BvhItem &y) {
+                             return x.c[ax] < y.c[ax] || (x.c[ax] == y.c[ax] && x.t < y.t);
+                         });
+        const int l = (int)next;
+        nd.left = l;
+        const int64_t next_l = next + 2, next_r = next_l + size(mid - lo) - 1;
+        std::thread th;
+        if (n >= 2 * THREAD_MIN) {
+            try {
+                th = std::thread([=] { build(l, lo, mid, next_l); });
+            } catch (const std::exception &) {
+                // no thread to be had: build it here
+            }
+        }
+        if (!th.joinable()) build(l, lo, mid, next_l);
+        build(l + 1, mid, hi, next_r);
+        if (th.joinable()) th.join();
     }
+};
+
+static void build_bvh(const double *V, const int32_t *T, int64_t nt, BvhBuilder &B)
+{
+    B.items.resize(nt);
+    B.order.resize(nt);
+    B.nodes.resize(BvhBuilder::size(nt));
+    for (int64_t t = 0; t < nt; ++t) {
+        for (int a = 0; a < 3; ++a) {
+            const double x0 = V[3 * (int64_t)T[3 * t] + a], x1 = V[3 * (int64_t)T[3 * t + 1] + a], x2 = V[3 * (int64_t)T[3 * t + 2] + a];
+            B.items[t].c[a] = 0.5 * (std::min(x0, std::min(x1, x2)) + std::max(x0, std::max(x1, x2)));
+        }
+        B.items[t].t = (int32_t)t;
+    }
+    B.build(0, 0, (int)nt, 1);
 }
 
 extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int64_t V, const int32_t *tris, int64_t T,
@@ -855,64 +792,81 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     for (int a = 0; a < 3; ++a) d3[a] = (int)ceil(((double)(N - 1) * h) / cs) + 1;
     d2[0] = d3[1];
     d2[1] = d3[2];
-    std::vector<int32_t> s3, i3, s2, i2;
-    build_bins3(verts, tris, T, ob->o, cs, d3, cut, s3, i3);
-    build_bins2(verts, tris, T, ob->o, cs, d2, s2, i2);
-    // device buffers
-    double *dV = nullptr;
-    float *dVf = nullptr, *dsph = nullptr;
-    int32_t *dorder = nullptr;
-    BvhNode *dnodes = nullptr;
-    size_t n_dnodes = 0;
-    int32_t *dT = nullptr, *ds3 = nullptr, *di3 = nullptr, *ds2 = nullptr, *di2 = nullptr;
-    uint8_t *dtouch = nullptr;
-    double2 *w1 = nullptr, *w2 = nullptr;
-    size_t tmp_bytes = 0;
+    // per axis, the first voxel index whose cell is >= c
+    std::vector<int32_t> axis;
+    for (int a = 0; a < 3; ++a) {
+        int k = 0;
+        for (int c = 0; c < d3[a]; ++c) {
+            while (k < N && (int)floor(((h * (double)k + ob->o[a]) - ob->o[a]) / cs) < c) ++k;
+            axis.push_back(k);
+        }
+        axis.push_back(N);
+    }
+    const size_t n3 = (size_t)d3[0] * d3[1] * d3[2], n2 = (size_t)d2[0] * d2[1];
+    // temporary device buffers, released together
+    struct Tmp { void *p; size_t bytes; };
+    std::vector<Tmp> tmp;
     auto cleanup_tmp = [&]() {
-        dfree(ctx, dV, sizeof(double) * 3 * V);
-        dfree(ctx, dVf, sizeof(float) * 3 * V);
-        dfree(ctx, dsph, sizeof(float) * 4 * T);
-        dfree(ctx, dorder, sizeof(int32_t) * T);
-        dfree(ctx, dnodes, sizeof(BvhNode) * n_dnodes);
-        dfree(ctx, dT, sizeof(int32_t) * 3 * T);
-        dfree(ctx, ds3, sizeof(int32_t) * s3.size());
-        dfree(ctx, di3, sizeof(int32_t) * i3.size());
-        dfree(ctx, ds2, sizeof(int32_t) * s2.size());
-        dfree(ctx, di2, sizeof(int32_t) * i2.size());
-        dfree(ctx, dtouch, (size_t)T);
-        dfree(ctx, w1, sizeof(double2) * (size_t)N * N * (N + 1));
-        dfree(ctx, w2, sizeof(double2) * (size_t)N * M * (N + 1));
+        for (auto &t : tmp) dfree(ctx, t.p, t.bytes);
+        tmp.clear();
     };
     auto bail = [&](dock_status st) {
         cleanup_tmp();
         dock_object_free(ob);
         return st;
     };
-    if ((s = dalloc(ctx, (void **)&dV, sizeof(double) * 3 * V, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&dT, sizeof(int32_t) * 3 * T, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ds3, sizeof(int32_t) * s3.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&di3, sizeof(int32_t) * i3.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ds2, sizeof(int32_t) * s2.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&di2, sizeof(int32_t) * i2.size(), &tmp_bytes)) != DOCK_OK) return bail(s);
-    if (touchable && (s = dalloc(ctx, (void **)&dtouch, (size_t)T, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->O, sizeof(float) * (size_t)N * N * N, &ob->bytes)) != DOCK_OK) return bail(s);
-    size_t spec_n = (size_t)M * P / 32 * M * 32;
-    if ((s = dalloc(ctx, (void **)&ob->spec, sizeof(float2) * spec_n, &ob->bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->o_dev, sizeof(double) * 3, &ob->bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&w1, sizeof(double2) * (size_t)N * N * (N + 1), &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&w2, sizeof(double2) * (size_t)N * M * (N + 1), &tmp_bytes)) != DOCK_OK) return bail(s);
+    auto temp = [&](void *pp, size_t bytes) -> dock_status {
+        void *q = nullptr;
+        const dock_status r = dalloc(ctx, &q, bytes, nullptr);
+        if (r == DOCK_OK) tmp.push_back({q, bytes});
+        *static_cast<void **>(pp) = q;
+        return r;
+    };
+    double *dV = nullptr;
+    int32_t *dT = nullptr, *ds3 = nullptr, *di3 = nullptr, *ds2 = nullptr, *di2 = nullptr, *at3 = nullptr, *at2 = nullptr;
+    int32_t *dorder = nullptr, *dwhich = nullptr, *daxis = nullptr;
+    BvhNode *dnodes = nullptr;
+    void *dtri = nullptr;
+    uint32_t *dinside = nullptr;
+    uint8_t *dtouch = nullptr;
+    double2 *w1 = nullptr, *w2 = nullptr;
     cudaStream_t st = ctx->stream;
 #define CKB(call)                                                   \
     do {                                                            \
         cudaError_t e_ = (call);                                    \
         if (e_ != cudaSuccess) return bail(cuda_fail(ctx, e_, #call)); \
     } while (0)
+    if ((s = temp(&dV, sizeof(double) * 3 * V)) != DOCK_OK) return bail(s);
+    if ((s = temp(&dT, sizeof(int32_t) * 3 * T)) != DOCK_OK) return bail(s);
+    if ((s = temp(&ds3, sizeof(int32_t) * 2 * (n3 + 1 + n2 + 1))) != DOCK_OK) return bail(s);
+    ds2 = ds3 + n3 + 1;
+    at3 = ds2 + n2 + 1;
+    at2 = at3 + n3 + 1;
     CKB(cudaMemcpyAsync(dV, verts, sizeof(double) * 3 * V, cudaMemcpyHostToDevice, st));
     CKB(cudaMemcpyAsync(dT, tris, sizeof(int32_t) * 3 * T, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(ds3, s3.data(), sizeof(int32_t) * s3.size(), cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(di3, i3.data(), sizeof(int32_t) * i3.size(), cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(ds2, s2.data(), sizeof(int32_t) * s2.size(), cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(di2, i2.data(), sizeof(int32_t) * i2.size(), cudaMemcpyHostToDevice, st));
+    CKB(cudaMemsetAsync(ds3, 0, sizeof(int32_t) * (n3 + 1 + n2 + 1), st));
+    CKB(launch_bins_count(dV, dT, T, ob->o, cs, d3, false, cut, ds3, st));
+    CKB(launch_bins_count(dV, dT, T, ob->o, cs, d3, true, 0.0, ds2, st));
+    CKB(cudaMemcpyAsync(at3, ds3, sizeof(int32_t) * (n3 + 1 + n2 + 1), cudaMemcpyDeviceToDevice, st));
+    int32_t total3 = 0, total2 = 0;
+    CKB(cudaMemcpyAsync(&total3, ds3 + n3, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CKB(cudaMemcpyAsync(&total2, ds2 + n2, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CKB(cudaStreamSynchronize(st));
+    if ((s = temp(&di3, sizeof(int32_t) * std::max(1, total3))) != DOCK_OK) return bail(s);
+    if ((s = temp(&di2, sizeof(int32_t) * std::max(1, total2))) != DOCK_OK) return bail(s);
+    if ((s = temp(&dtri, tri_f32_bytes() * T)) != DOCK_OK) return bail(s);
+    if ((s = temp(&dinside, sizeof(uint32_t) * (size_t)N * N * (N / 32))) != DOCK_OK) return bail(s);
+    if ((s = temp(&daxis, sizeof(int32_t) * axis.size())) != DOCK_OK) return bail(s);
+    if (touchable && (s = temp(&dtouch, (size_t)T)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&ob->O, sizeof(float) * (size_t)N * N * N, &ob->bytes)) != DOCK_OK) return bail(s);
+    size_t spec_n = (size_t)M * P / 32 * M * 32;
+    if ((s = dalloc(ctx, (void **)&ob->spec, sizeof(float2) * spec_n, &ob->bytes)) != DOCK_OK) return bail(s);
+    if ((s = dalloc(ctx, (void **)&ob->o_dev, sizeof(double) * 3, &ob->bytes)) != DOCK_OK) return bail(s);
+    if ((s = temp(&w1, sizeof(double2) * (size_t)N * N * (N + 1))) != DOCK_OK) return bail(s);
+    if ((s = temp(&w2, sizeof(double2) * (size_t)N * M * (N + 1))) != DOCK_OK) return bail(s);
+    CKB(launch_bins_fill(dV, dT, T, ob->o, cs, d3, false, cut, at3, di3, st));
+    CKB(launch_bins_fill(dV, dT, T, ob->o, cs, d3, true, 0.0, at2, di2, st));
+    CKB(cudaMemcpyAsync(daxis, axis.data(), sizeof(int32_t) * axis.size(), cudaMemcpyHostToDevice, st));
     if (dtouch) CKB(cudaMemcpyAsync(dtouch, touchable, (size_t)T, cudaMemcpyHostToDevice, st));
     CKB(cudaMemcpyAsync(ob->o_dev, ob->o, sizeof(double) * 3, cudaMemcpyHostToDevice, st));
     CKB(cudaMemsetAsync(ctx->errflag, 0, sizeof(int), st));
@@ -927,36 +881,35 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     bins.cs = cs;
     {
         Prof pr(ctx, "object_grid");
-        CKB(launch_object_grid(dV, dT, dtouch, bins, N, h, ob->o, p->tau_out1, p->tau_in1, p->deep_value, ob->O,
-                               nullptr, ctx->errflag, st));
+        CKB(launch_object_grid(dV, dT, T, dtouch, bins, daxis, N, h, ob->o, p->tau_out1, p->tau_in1, p->deep_value, dtri,
+                               dinside, ob->O, ctx->errflag, st));
     }
     {
         Prof pr(ctx, "object_spectrum");
         CKB(launch_spectrum(ob->O, N, M, P, w1, w2, twd, ob->spec, st));
     }
-    // mesh + BVH for the refinement
-    std::vector<BvhNode> nodes;
-    std::vector<int32_t> order;
-    std::vector<float> tsph;
-    build_bvh(verts, tris, T, nodes, order, tsph);
-    std::vector<float> vf(3 * V);
-    for (int64_t i = 0; i < 3 * V; ++i) vf[i] = (float)verts[i];
+    // the tree of the refinement, beside the kernels above
+    BvhBuilder bvh;
+    build_bvh(verts, tris, T, bvh);
+    const size_t nn = bvh.nodes.size();
+    std::vector<int32_t> which;
+    which.reserve(nn);
+    for (size_t i = 0; i < nn; ++i) if (bvh.nodes[i].count > BVH_BIG) which.push_back((int32_t)i);
+    const int n_big = (int)which.size();
+    for (size_t i = 0; i < nn; ++i) if (bvh.nodes[i].count <= BVH_BIG) which.push_back((int32_t)i);
     ob->nv = V;
     ob->nt = T;
-    ob->n_nodes = (int)nodes.size();
-    if ((s = dalloc(ctx, (void **)&dVf, sizeof(float) * 3 * V, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&dsph, sizeof(float) * 4 * T, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&dorder, sizeof(int32_t) * T, &tmp_bytes)) != DOCK_OK) return bail(s);
+    ob->n_nodes = (int)nn;
+    if ((s = temp(&dorder, sizeof(int32_t) * T)) != DOCK_OK) return bail(s);
+    if ((s = temp(&dnodes, sizeof(BvhNode) * nn)) != DOCK_OK) return bail(s);
+    if ((s = temp(&dwhich, sizeof(int32_t) * nn)) != DOCK_OK) return bail(s);
     if ((s = dalloc(ctx, (void **)&ob->leaf, leaf_bytes() * T, &ob->bytes)) != DOCK_OK) return bail(s);
-    n_dnodes = nodes.size();
-    if ((s = dalloc(ctx, (void **)&dnodes, sizeof(BvhNode) * n_dnodes, &tmp_bytes)) != DOCK_OK) return bail(s);
-    if ((s = dalloc(ctx, (void **)&ob->nodes, node_bytes() * n_dnodes, &ob->bytes)) != DOCK_OK) return bail(s);
-    CKB(cudaMemcpyAsync(dVf, vf.data(), sizeof(float) * 3 * V, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(dsph, tsph.data(), sizeof(float) * 4 * T, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(dorder, order.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
-    CKB(cudaMemcpyAsync(dnodes, nodes.data(), sizeof(BvhNode) * nodes.size(), cudaMemcpyHostToDevice, st));
-    CKB(launch_leaf_records((int)T, dVf, dT, dsph, dorder, ob->leaf, st));
-    CKB(launch_node_records((int)n_dnodes, dnodes, ob->leaf, ob->nodes, st));
+    if ((s = dalloc(ctx, (void **)&ob->nodes, node_bytes() * nn, &ob->bytes)) != DOCK_OK) return bail(s);
+    CKB(cudaMemcpyAsync(dorder, bvh.order.data(), sizeof(int32_t) * T, cudaMemcpyHostToDevice, st));
+    CKB(cudaMemcpyAsync(dnodes, bvh.nodes.data(), sizeof(BvhNode) * nn, cudaMemcpyHostToDevice, st));
+    CKB(cudaMemcpyAsync(dwhich, which.data(), sizeof(int32_t) * nn, cudaMemcpyHostToDevice, st));
+    CKB(launch_leaf_records((int)T, dV, dT, dorder, ob->leaf, st));
+    CKB(launch_node_records((int)nn, n_big, dwhich, dnodes, dV, dT, dorder, ob->leaf, ob->nodes, st));
     int herr = 0;
     CKB(cudaMemcpyAsync(&herr, ctx->errflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     CKB(cudaStreamSynchronize(st));

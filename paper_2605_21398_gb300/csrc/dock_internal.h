@@ -147,6 +147,13 @@ cudaError_t launch_vox_float(const Geo &g, const ReqDev *reqs, const RotRec *rot
 cudaError_t launch_rot_export(const Geo &g, const ReqDev *reqs, const RotRec *rots, int B, float *out, cudaStream_t st);
 
 // Object grid kernels (k_object.cu)
+// Bins of triangles over cells of side cs, CSR: per triangle the cells its box
+// (widened by pad) meets; cells over (x, y, z), or over (y, z) when flat.  count: n_cells + 1 zeros in, exclusive prefix sums out (the total at
+// the end); fill writes the items, `at` being a copy of the prefix sums.
+cudaError_t launch_bins_count(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                              bool flat, double pad, int32_t *start, cudaStream_t st);
+cudaError_t launch_bins_fill(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                             bool flat, double pad, int32_t *at, int32_t *items, cudaStream_t st);
 struct ObjBins {
     const int32_t *cell3_start;  // 3-D cells, CSR
     const int32_t *cell3_items;
@@ -156,9 +163,13 @@ struct ObjBins {
     int d2[2];
     double cs;                    // cell size
 };
-cudaError_t launch_object_grid(const double *V, const int32_t *T, const uint8_t *touch, const ObjBins &bins,
-                               int N, double h, const double *o, double tau_out, double tau_in, double deep,
-                               float *O, float *f_out, int *err, cudaStream_t st);
+// axis: per axis, the first voxel index whose cell is >= c (d3 + 1 entries
+// each); tri: nt records of tri_f32_bytes(); inside: N^3 bits (both workspaces)
+size_t tri_f32_bytes();
+cudaError_t launch_object_grid(const double *V, const int32_t *T, int64_t nt, const uint8_t *touch, const ObjBins &bins,
+                               const int32_t *axis, int N, double h, const double *o, double tau_out, double tau_in,
+                               double deep, void *tri, uint32_t *inside, float *O, int *err, cudaStream_t st);
+// The canvas spectrum (k_spectrum.cu).
 // pen: transform min(O, 0) instead of O (the label-aware penetration part).
 // conj = false stores F(O) / M^3 (the fixed swept grid of rotate_object).
 cudaError_t launch_spectrum(const float *O, int N, int M, int P, double2 *work1, double2 *work2,
@@ -166,20 +177,23 @@ cudaError_t launch_spectrum(const float *O, int N, int M, int P, double2 *work1,
 
 // Refinement kernels (k_refine.cu)
 struct BvhNode {
-    float c[3];    // sphere centre (object frame)
-    float rad;     // sphere radius
-    int32_t left;  // child index, or -1 for a leaf
-    int32_t right; // right child (left + 1), or the leaf's first slot in the triangle order
+    int32_t left;  // child index (the right child is the next node), or -1 for a leaf
+    int32_t first; // first slot of its triangles in the leaf order
     int32_t count; // triangles below the node
-    int32_t pad;   // interior node: first slot of its triangles
+    int32_t pad;
 };
+constexpr int BVH_BIG = 2048;   // nodes of more triangles are finished by a block instead of a warp
 struct LeafRec;               // one triangle of a leaf (k_refine.cu)
 struct NodeRec;               // one BVH node (k_refine.cu)
 size_t leaf_bytes();
 size_t node_bytes();
-cudaError_t launch_node_records(int n, const BvhNode *in, const LeafRec *leaf, NodeRec *out, cudaStream_t st);
-cudaError_t launch_leaf_records(int n, const float *Vf, const int32_t *T, const float *tri_sphere,
-                                const int32_t *tri_order, LeafRec *out, cudaStream_t st);
+// The device records of the n nodes and of the triangles in leaf order.  big: the
+// indices of the n_big nodes of more than BVH_BIG triangles, then the others'.
+cudaError_t launch_node_records(int n, int n_big, const int32_t *big, const BvhNode *in, const double *V,
+                                const int32_t *T, const int32_t *order, const LeafRec *leaf, NodeRec *out,
+                                cudaStream_t st);
+cudaError_t launch_leaf_records(int n, const double *V, const int32_t *T, const int32_t *order, LeafRec *out,
+                                cudaStream_t st);
 struct RefineDev {
     const LeafRec *leaf;      // triangles in leaf order
     const NodeRec *nodes;

@@ -1,4 +1,4 @@
-// Object grid (Sec. IV-A.1, Eq. (1)-(4)) and its canvas spectrum (Eq. (9)).
+// Object grid (Sec. IV-A.1, Eq. (1)-(4)).
 //
 // This translation unit is compiled with -fmad=false: every FP64 expression
 // is rounded exactly as written, so the signed distance, its sign and the band
@@ -72,11 +72,103 @@ __device__ int edge_side(double ay, double az, double by, double bz, double py, 
     return 0;
 }
 
-// One block per lattice row (ky, kz); thread kx.  The row's crossings with
-// the mesh along +x decide the sign (odd count beyond x = inside).
-__global__ void k_object_grid(const double *V, const int32_t *T, const uint8_t *touch, ObjBins bins, int N, double h,
-                              double o0, double o1, double o2, double tau_out, double tau_in, double deep, float *O,
-                              float *f_out, int *err)
+// The cells triangle t's box meets, per axis (axis 0 is y when flat); false when none.
+__device__ __forceinline__ bool tri_cells(const double *V, const int32_t *T, int64_t t, const double3 o, double cs,
+                                          const int3 d, bool flat, double pad, int *lo, int *hi)
+{
+    const double org[3] = {o.x, o.y, o.z};
+    const int dim[3] = {d.x, d.y, d.z};
+    for (int a = flat ? 1 : 0; a < 3; ++a) {
+        const double x0 = V[3 * (size_t)T[3 * t] + a], x1 = V[3 * (size_t)T[3 * t + 1] + a], x2 = V[3 * (size_t)T[3 * t + 2] + a];
+        const double mn = fmin(x0, fmin(x1, x2)) - pad, mx = fmax(x0, fmax(x1, x2)) + pad;
+        const double l = floor((mn - org[a]) / cs), h = floor((mx - org[a]) / cs);
+        lo[a] = l > 0.0 ? (l < (double)dim[a] ? (int)l : dim[a]) : 0;
+        hi[a] = h < (double)(dim[a] - 1) ? (h >= 0.0 ? (int)h : -1) : dim[a] - 1;
+        if (lo[a] > hi[a]) return false;
+    }
+    if (flat) lo[0] = hi[0] = 0;
+    return true;
+}
+
+// at[cell] += 1 per triangle and cell; with items given, the old value is the
+// triangle's place (the order within a cell does not matter: minima and
+// parities are taken over it)
+__global__ void k_bins(const double *V, const int32_t *T, int64_t nt, double3 o, double cs, int3 d, bool flat, double pad,
+                       int32_t *at, int32_t *items)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nt) return;
+    int lo[3], hi[3];
+    if (!tri_cells(V, T, t, o, cs, d, flat, pad, lo, hi)) return;
+    const int w = flat ? 1 : d.x;
+    for (int z = lo[2]; z <= hi[2]; ++z)
+        for (int y = lo[1]; y <= hi[1]; ++y)
+            for (int x = lo[0]; x <= hi[0]; ++x) {
+                const int64_t c = ((int64_t)z * d.y + y) * w + x;
+                const int k = atomicAdd(&at[c], 1);
+                if (items) items[k] = (int32_t)t;
+            }
+}
+
+// exclusive prefix sums of n counts in place (one block); at[n] gets the total
+__global__ void __launch_bounds__(1024) k_bins_scan(int32_t *at, int n)
+{
+    __shared__ int32_t warp_sum[32];
+    __shared__ int32_t carry;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) carry = 0;
+    __syncthreads();
+    for (int base = 0; base < n; base += 1024) {
+        const int i = base + tid;
+        const int32_t v = i < n ? at[i] : 0;
+        int32_t x = v;
+        for (int s = 1; s < 32; s <<= 1) {
+            const int32_t y = __shfl_up_sync(0xFFFFFFFFu, x, s);
+            if (lane >= s) x += y;
+        }
+        if (lane == 31) warp_sum[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            int32_t w = warp_sum[lane];
+            for (int s = 1; s < 32; s <<= 1) {
+                const int32_t y = __shfl_up_sync(0xFFFFFFFFu, w, s);
+                if (lane >= s) w += y;
+            }
+            warp_sum[lane] = w;
+        }
+        __syncthreads();
+        const int32_t before = carry + (warp ? warp_sum[warp - 1] : 0) + x - v;
+        if (i < n) at[i] = before;
+        __syncthreads();
+        if (tid == 1023) carry = before + v;
+        __syncthreads();
+    }
+    if (tid == 0) at[n] = carry;
+}
+
+cudaError_t launch_bins_count(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                              bool flat, double pad, int32_t *start, cudaStream_t st)
+{
+    k_bins<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>(V, T, nt, make_double3(o[0], o[1], o[2]), cs,
+                                                         make_int3(d[0], d[1], d[2]), flat, pad, start, nullptr);
+    k_bins_scan<<<1, 1024, 0, st>>>(start, (flat ? 1 : d[0]) * d[1] * d[2]);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bins_fill(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                             bool flat, double pad, int32_t *at, int32_t *items, cudaStream_t st)
+{
+    k_bins<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>(V, T, nt, make_double3(o[0], o[1], o[2]), cs,
+                                                         make_int3(d[0], d[1], d[2]), flat, pad, at, items);
+    return cudaGetLastError();
+}
+
+// One block per lattice row (ky, kz); thread kx < N.  The row's crossings with
+// the mesh along +x decide the sign (odd count beyond x = inside): inside[row]
+// gets one bit per voxel.
+__global__ void __launch_bounds__(128)
+k_object_rows(const double *V, const int32_t *T, ObjBins bins, int N, double h, double o0, double o1, double o2,
+              uint32_t *inside, int *err)
 {
     __shared__ double xs[1024];
     __shared__ int nx;
@@ -107,126 +199,229 @@ __global__ void k_object_grid(const double *V, const int32_t *T, const uint8_t *
         }
     }
     __syncthreads();
-    const int n_cross = min(nx, 1024);
+    const int n_cross = min(nx, 1024), kx = threadIdx.x;
+    if (kx >= N) return;   // whole warps: N is a multiple of 32
+    const double p0 = h * (double)kx + o0;
+    int par = 0;
+    for (int c = 0; c < n_cross; ++c) par ^= (xs[c] > p0) ? 1 : 0;
+    const uint32_t w = __ballot_sync(0xFFFFFFFFu, par);
+    if ((kx & 31) == 0) inside[(size_t)blockIdx.x * (N / 32) + kx / 32] = w;
+}
+
+// A triangle in FP32 relative to the lattice origin: v0, the edges to v1 and
+// v2, its longest edge, and how far (mm) an FP32 distance to it may be off.
+struct TriF {
+    float v0[3], e0[3], e1[3], reach, tol;
+    int32_t touch;
+};
+static_assert(sizeof(TriF) == 48, "triangle record");
+
+size_t tri_f32_bytes() { return sizeof(TriF); }
+
+// S: the lattice's extent; a coordinate relative to its origin is rounded to
+// 2^-24 S (point and vertex).  A normal of a triangle of altitude a turns by
+// that over a, which moves a plane distance measured from up to 2 cut + edge
+// away; degenerate triangles get an infinite tolerance.
+__global__ void k_tri_f32(int n, const double *V, const int32_t *T, const uint8_t *touch, double o0, double o1,
+                          double o2, float S, float cut, TriF *out)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const double o[3] = {o0, o1, o2};
+    float v[3][3];
+    for (int m = 0; m < 3; ++m)
+        for (int a = 0; a < 3; ++a) v[m][a] = (float)(V[3 * (size_t)T[3 * t + m] + a] - o[a]);
+    TriF r;
+    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
+    for (int a = 0; a < 3; ++a) {
+        r.v0[a] = v[0][a];
+        r.e0[a] = v[1][a] - v[0][a];
+        r.e1[a] = v[2][a] - v[0][a];
+        const float d = v[2][a] - v[1][a];
+        l0 += r.e0[a] * r.e0[a];
+        l1 += r.e1[a] * r.e1[a];
+        l2 += d * d;
+    }
+    const float n0 = r.e0[1] * r.e1[2] - r.e0[2] * r.e1[1], n1 = r.e0[2] * r.e1[0] - r.e0[0] * r.e1[2];
+    const float n2 = r.e0[0] * r.e1[1] - r.e0[1] * r.e1[0];
+    const float edge = sqrtf(fmaxf(l0, fmaxf(l1, l2))), area = sqrtf(n0 * n0 + n1 * n1 + n2 * n2);
+    const float delta = 5e-7f * S, far = 2.f * cut + edge;
+    // the altitude itself is uncertain by a few delta
+    const float alt = edge > 0.f ? area / edge - 8.f * delta : 0.f;
+    r.reach = edge + 4.f * delta;
+    r.tol = alt > 0.f ? 4.f * delta * (1.f + far / alt) : INFINITY;
+    r.touch = (touch == nullptr || touch[t]) ? 1 : 0;
+    out[t] = r;
+}
+
+// FP32 distance from p (relative to the lattice origin) to a triangle: the
+// smallest of the three edges' and, when the projection falls inside, the
+// plane's.  INFINITY when farther than `skip` (a bound on what matters).
+__device__ __forceinline__ float tri_dist_f32(const TriF &t, float px, float py, float pz, float skip)
+{
+    const float w0 = px - t.v0[0], w1 = py - t.v0[1], w2 = pz - t.v0[2];
+    const float ww = fmaf(w0, w0, fmaf(w1, w1, w2 * w2)), lim = skip + t.reach;
+    if (ww > lim * lim) return INFINITY;
+    const float *a = t.e0, *b = t.e1;
+    const float aa = fmaf(a[0], a[0], fmaf(a[1], a[1], a[2] * a[2])), bb = fmaf(b[0], b[0], fmaf(b[1], b[1], b[2] * b[2]));
+    const float ab = fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2]));
+    const float wa = fmaf(w0, a[0], fmaf(w1, a[1], w2 * a[2])), wb = fmaf(w0, b[0], fmaf(w1, b[1], w2 * b[2]));
+    // nearest point of each edge: w - t e
+    auto off = [&](float s, float u) -> float {   // |w - s a - u b|^2
+        const float q0 = w0 - fmaf(s, a[0], u * b[0]), q1 = w1 - fmaf(s, a[1], u * b[1]), q2 = w2 - fmaf(s, a[2], u * b[2]);
+        return fmaf(q0, q0, fmaf(q1, q1, q2 * q2));
+    };
+    const float sa = aa > 0.f ? fminf(1.f, fmaxf(0.f, wa / aa)) : 0.f;
+    const float sb = bb > 0.f ? fminf(1.f, fmaxf(0.f, wb / bb)) : 0.f;
+    // edge v1 v2: points (1 - s) a + s b
+    const float cc = aa - 2.f * ab + bb, wc = (wb - wa) - (ab - aa);
+    const float sc = cc > 0.f ? fminf(1.f, fmaxf(0.f, wc / cc)) : 0.f;
+    float d2 = fminf(off(sa, 0.f), fminf(off(0.f, sb), off(1.f - sc, sc)));
+    const float den = fmaf(aa, bb, -ab * ab), u = fmaf(bb, wa, -ab * wb), v = fmaf(aa, wb, -ab * wa);
+    if (den > 0.f && u >= 0.f && v >= 0.f && u + v <= den) {
+        const float n0 = a[1] * b[2] - a[2] * b[1], n1 = a[2] * b[0] - a[0] * b[2], n2 = a[0] * b[1] - a[1] * b[0];
+        const float nn = fmaf(n0, n0, fmaf(n1, n1, n2 * n2)), wn = fmaf(w0, n0, fmaf(w1, n1, w2 * n2));
+        if (nn > 0.f) d2 = fminf(d2, wn * wn / nn);
+    }
+    return sqrtf(d2);
+}
+
+// One block per bin cell: band values of the cell's voxels.  FP64 operations
+// run at a 64th of the FP32 rate, so the triangles of the cell (about 500 near
+// a surface of 65 k triangles) are measured in FP32 first, and the exact FP64
+// distance (whose minimum is the result) is formed only for those that the FP32
+// distance and its error bound leave in question, a few per voxel.  Two
+// threads per voxel share the triangles of a tile; the voxel-triangle pairs in
+// question are dealt to the block.  44.2 -> 3.1 ms (rows and cells) at N = 128 and 65 k triangles
+// (with one thread per voxel and FP64 throughout, lanes of a warp walking
+// different cells).
+// axis[a][c]: first voxel index along axis a whose cell is >= c (d3[a] + 1 entries
+// each, the axes one after another).
+__global__ void __launch_bounds__(128)
+k_object_cells(const double *V, const int32_t *T, const TriF *tri, ObjBins bins, const int32_t *axis, int N, double h,
+               double o0, double o1, double o2, double tau_out, double tau_in, double deep, const uint32_t *inside,
+               float *O)
+{
+    constexpr int NT = 128, NV = 64, TILE = 64, PAIRS = 4096, ROOM = 8 * NT;
+    __shared__ TriF tile[TILE];
+    __shared__ int tidx[TILE];
+    __shared__ unsigned long long best[NV], bestt[NV];
+    __shared__ int pair_i[PAIRS];             // item of the cell's list
+    __shared__ unsigned char pair_s[PAIRS];   // voxel slot
+    __shared__ int n_pairs;
+    const int tid = threadIdx.x;
+    const int cx = blockIdx.x % bins.d3[0], cy = (blockIdx.x / bins.d3[0]) % bins.d3[1], cz = blockIdx.x / (bins.d3[0] * bins.d3[1]);
+    const int32_t *ax = axis, *ay = ax + bins.d3[0] + 1, *az = ay + bins.d3[1] + 1;
+    const int x0 = ax[cx], y0 = ay[cy], z0 = az[cz], lx = ax[cx + 1] - x0, ly = ay[cy + 1] - y0, lz = az[cz + 1] - z0;
+    const int nv = lx * ly * lz;
+    const int i0 = bins.cell3_start[blockIdx.x], n_items = bins.cell3_start[blockIdx.x + 1] - i0;
+    const double cut = tau_out > tau_in ? tau_out : tau_in, cut2 = cut * cut;
+    const float skip = (float)cut * 1.00001f;
+    // exact distances of the pairs in question
+    auto settle = [&](int base) {
+        __syncthreads();
+        const int np = n_pairs;
+        for (int k = tid; k < np; k += NT) {
+            const int s = pair_s[k], t = bins.cell3_items[i0 + pair_i[k]], v = base + s;
+            const double p[3] = {h * (double)(x0 + v % lx) + o0, h * (double)(y0 + (v / lx) % ly) + o1,
+                                 h * (double)(z0 + v / (lx * ly)) + o2};
+            const double d2 = tri_dist2(p, V + 3 * (size_t)T[3 * t], V + 3 * (size_t)T[3 * t + 1], V + 3 * (size_t)T[3 * t + 2]);
+            // distances are not negative: their bits are in their order (a NaN never is the smallest)
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(d2);
+            atomicMin(&best[s], bits);
+            if (tri[t].touch) atomicMin(&bestt[s], bits);
+        }
+        __syncthreads();
+        if (tid == 0) n_pairs = 0;
+        __syncthreads();
+    };
+    for (int base = 0; base < nv; base += NV) {
+        const int s = tid >> 1, half = tid & 1, v = base + s;
+        const bool on = v < nv;
+        const float px = (float)(h * (double)(x0 + v % lx)), py = (float)(h * (double)(y0 + (v / lx) % ly));
+        const float pz = (float)(h * (double)(z0 + v / (lx * ly)));
+        if (tid < NV) best[tid] = bestt[tid] = 0x7FF0000000000000ull;   // +infinity
+        if (tid == 0) n_pairs = 0;
+        // pass 0: upper bounds of the two minima; pass 1: the pairs in question
+        float ub = INFINITY, ubt = INFINITY;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+            for (int j0 = 0; j0 < n_items; j0 += TILE) {
+                const int nt = min(TILE, n_items - j0);
+                __syncthreads();
+                for (int k = tid; k < nt; k += NT) tidx[k] = bins.cell3_items[i0 + j0 + k];
+                __syncthreads();
+                for (int k = tid; k < nt * 12; k += NT)
+                    reinterpret_cast<uint32_t *>(tile)[k] = reinterpret_cast<const uint32_t *>(tri + tidx[k / 12])[k % 12];
+                __syncthreads();
+                for (int k0 = 0; k0 < nt; k0 += 16) {
+                    // eight triangles of the tile per thread, then room is looked for again
+                    if (on)
+                        for (int k = k0 + half; k < min(nt, k0 + 16); k += 2) {
+                            const TriF &t = tile[k];
+                            // (a triangle without a usable FP32 distance is always in question)
+                            const bool sure = t.tol < INFINITY;
+                            const float b = fminf(skip, fmaxf(ub, ubt));
+                            const float d = sure ? tri_dist_f32(t, px, py, pz, b + t.tol) : 0.f;
+                            if (pass == 0) {
+                                if (sure) {
+                                    ub = fminf(ub, d + t.tol);
+                                    if (t.touch) ubt = fminf(ubt, d + t.tol);
+                                }
+                            } else if (!sure || d - t.tol <= fminf(skip, ub) || (t.touch && d - t.tol <= fminf(skip, ubt))) {
+                                const int k2 = atomicAdd(&n_pairs, 1);
+                                pair_i[k2] = j0 + k;
+                                pair_s[k2] = (unsigned char)s;
+                            }
+                        }
+                    if (pass == 1) {
+                        __syncthreads();
+                        const bool full = n_pairs > PAIRS - ROOM;
+                        __syncthreads();
+                        if (full) settle(base);
+                    }
+                }
+            }
+            if (pass == 0) {
+                ub = fminf(ub, __shfl_xor_sync(0xFFFFFFFFu, ub, 1));
+                ubt = fminf(ubt, __shfl_xor_sync(0xFFFFFFFFu, ubt, 1));
+            }
+        }
+        settle(base);
+        if (tid < NV && base + tid < nv) {
+            const int vv = base + tid, kx = x0 + vv % lx, ky = y0 + (vv / lx) % ly, kz = z0 + vv / (lx * ly);
+            const size_t row = (size_t)kz * N + ky;
+            const int par = (inside[row * (N / 32) + kx / 32] >> (kx & 31)) & 1u;
+            const double b2 = __longlong_as_double((long long)best[tid]), bt2 = __longlong_as_double((long long)bestt[tid]);
+            double D = b2 < cut2 ? sqrt(b2) : INFINITY;
+            double Dt = bt2 < cut2 ? sqrt(bt2) : INFINITY;
+            double f = par ? -D : D;
+            double Ot;
+            if (0.0 <= f && f < tau_out) Ot = 1.0 - f / tau_out;          // Eq. (1), first branch
+            else if (-tau_in < f && f < 0.0) Ot = 1.0 + f / tau_in;      // shallow penetration
+            else if (f <= -tau_in) Ot = deep;                            // deep penetration
+            else Ot = 0.0;
+            double Om = 1.0 - Dt / tau_out;                              // Eq. (2)
+            if (!(Om > 0.0)) Om = 0.0;
+            double val = Ot < Om ? Ot : Om;                              // Eq. (3)
+            O[row * N + kx] = (float)val;
+        }
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_object_grid(const double *V, const int32_t *T, int64_t nt, const uint8_t *touch, const ObjBins &bins,
+                               const int32_t *axis, int N, double h, const double *o, double tau_out, double tau_in,
+                               double deep, void *tri, uint32_t *inside, float *O, int *err, cudaStream_t st)
+{
+    TriF *tf = static_cast<TriF *>(tri);
     const double cut = tau_out > tau_in ? tau_out : tau_in;
-    const double cut2 = cut * cut;
-    for (int kx = threadIdx.x; kx < N; kx += blockDim.x) {
-        double p[3] = {h * (double)kx + o0, py, pz};
-        int par = 0;
-        for (int c = 0; c < n_cross; ++c) par ^= (xs[c] > p[0]) ? 1 : 0;
-        int cx = (int)floor((p[0] - o0) / bins.cs);
-        int cyy = (int)floor((p[1] - o1) / bins.cs);
-        int czz = (int)floor((p[2] - o2) / bins.cs);
-        double best = INFINITY, bestt = INFINITY;
-        if (cx >= 0 && cx < bins.d3[0] && cyy >= 0 && cyy < bins.d3[1] && czz >= 0 && czz < bins.d3[2]) {
-            int cell = (czz * bins.d3[1] + cyy) * bins.d3[0] + cx;
-            for (int k = bins.cell3_start[cell]; k < bins.cell3_start[cell + 1]; ++k) {
-                int t = bins.cell3_items[k];
-                double d2 = tri_dist2(p, V + 3 * T[3 * t], V + 3 * T[3 * t + 1], V + 3 * T[3 * t + 2]);
-                if (d2 < best) best = d2;
-                if ((touch == nullptr || touch[t]) && d2 < bestt) bestt = d2;
-            }
-        }
-        double D = best < cut2 ? sqrt(best) : INFINITY;
-        double Dt = bestt < cut2 ? sqrt(bestt) : INFINITY;
-        double f = par ? -D : D;
-        double Ot;
-        if (0.0 <= f && f < tau_out) Ot = 1.0 - f / tau_out;          // Eq. (1), first branch
-        else if (-tau_in < f && f < 0.0) Ot = 1.0 + f / tau_in;      // shallow penetration
-        else if (f <= -tau_in) Ot = deep;                            // deep penetration
-        else Ot = 0.0;
-        double Om = 1.0 - Dt / tau_out;                              // Eq. (2)
-        if (!(Om > 0.0)) Om = 0.0;
-        double val = Ot < Om ? Ot : Om;                              // Eq. (3)
-        size_t idx = ((size_t)kz * N + ky) * N + kx;
-        O[idx] = (float)val;
-        if (f_out) f_out[idx] = (float)f;
-    }
-}
-
-cudaError_t launch_object_grid(const double *V, const int32_t *T, const uint8_t *touch, const ObjBins &bins, int N,
-                               double h, const double *o, double tau_out, double tau_in, double deep, float *O,
-                               float *f_out, int *err, cudaStream_t st)
-{
-    k_object_grid<<<N * N, 128, 0, st>>>(V, T, touch, bins, N, h, o[0], o[1], o[2], tau_out, tau_in, deep, O, f_out,
-                                         err);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// conj(F(O)) / M^3 on the zero-padded M^3 canvas, FP64 direct DFT per axis
-// (O occupies the corner [0, N)^3), stored as FP32 in the z-pass tile order.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ double2 cmuld(double2 a, double2 b)
-{
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-// A[z][y][kx] = sum_x O[z][y][x] w^(kx x), kx in [0, H]  (min(O, 0) when pen)
-__global__ void k_spec_x(const float *O, int N, int M, const double2 *tw, double2 *A, bool pen)
-{
-    const int H = M / 2;
-    const int row = blockIdx.x;   // z * N + y
-    const float *o = O + (size_t)row * N;
-    for (int kx = threadIdx.x; kx <= H; kx += blockDim.x) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int x = 0; x < N; ++x) {
-            double v = (double)o[x];
-            if (pen) v = fmin(v, 0.0);
-            if (v != 0.0) {
-                double2 w = tw[(kx * x) % M];
-                acc.x += v * w.x;
-                acc.y += v * w.y;
-            }
-        }
-        A[(size_t)row * (H + 1) + kx] = acc;
-    }
-}
-
-// B[z][ky][kx] = sum_y A[z][y][kx] w^(ky y)
-__global__ void k_spec_y(const double2 *A, int N, int M, const double2 *tw, double2 *Bo)
-{
-    const int H = M / 2;
-    const int z = blockIdx.y, ky = blockIdx.x;
-    for (int kx = threadIdx.x; kx <= H; kx += blockDim.x) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int y = 0; y < N; ++y) {
-            double2 a = A[((size_t)z * N + y) * (H + 1) + kx];
-            double2 r = cmuld(a, tw[(ky * y) % M]);
-            acc.x += r.x;
-            acc.y += r.y;
-        }
-        Bo[((size_t)z * M + ky) * (H + 1) + kx] = acc;
-    }
-}
-
-// spec tile: conj(sum_z B[z][ky][kx] w^(kz z)) / M^3 at f = ky P + kx (no conj when !cj)
-__global__ void k_spec_z(const double2 *Bi, int N, int M, int P, const double2 *tw, float2 *spec, bool cj)
-{
-    const int H = M / 2;
-    const int ky = blockIdx.y, kz = blockIdx.x;
-    const double sc = 1.0 / ((double)M * (double)M * (double)M);
-    for (int kx = threadIdx.x; kx < P; kx += blockDim.x) {
-        double2 acc = make_double2(0.0, 0.0);
-        if (kx <= H) {
-            for (int z = 0; z < N; ++z) {
-                double2 r = cmuld(Bi[((size_t)z * M + ky) * (H + 1) + kx], tw[(kz * z) % M]);
-                acc.x += r.x;
-                acc.y += r.y;
-            }
-        }
-        size_t f = (size_t)ky * P + kx;
-        size_t chunk = f / 32, lane = f % 32;
-        spec[(chunk * M + kz) * 32 + lane] = make_float2((float)(acc.x * sc), (float)((cj ? -acc.y : acc.y) * sc));
-    }
-}
-
-cudaError_t launch_spectrum(const float *O, int N, int M, int P, double2 *work1, double2 *work2, const double2 *twd,
-                            float2 *spec, cudaStream_t st, bool pen, bool conj)
-{
-    k_spec_x<<<N * N, 160, 0, st>>>(O, N, M, twd, work1, pen);
-    k_spec_y<<<dim3(M, N), 160, 0, st>>>(work1, N, M, twd, work2);
-    k_spec_z<<<dim3(M, M), 160, 0, st>>>(work2, N, M, P, twd, spec, conj);
+    k_tri_f32<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>((int)nt, V, T, touch, o[0], o[1], o[2], (float)(N * h),
+                                                            (float)cut, tf);
+    k_object_rows<<<N * N, 128, 0, st>>>(V, T, bins, N, h, o[0], o[1], o[2], inside, err);
+    k_object_cells<<<bins.d3[0] * bins.d3[1] * bins.d3[2], 128, 0, st>>>(V, T, tf, bins, axis, N, h, o[0], o[1], o[2],
+                                                                        tau_out, tau_in, deep, inside, O);
     return cudaGetLastError();
 }
 

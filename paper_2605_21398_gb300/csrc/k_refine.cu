@@ -542,81 +542,145 @@ static_assert(sizeof(NodeRec) == 48, "node record");
 
 size_t node_bytes() { return sizeof(NodeRec); }
 
-// One warp per node over its triangles (interior nodes: right = first slot of
-// the range, count = its length, as built).
-__global__ void k_node_records(int n, const BvhNode *in, const LeafRec *leaf, NodeRec *out)
+// Bounding sphere of points given one by one (FP64, every operation rounded as
+// written): the centre of their box, the largest distance with a small pad.
+struct BoxD {
+    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+    __device__ __forceinline__ void add(const double *v)
+    {
+        for (int a = 0; a < 3; ++a) { lo[a] = fmin(lo[a], v[a]); hi[a] = fmax(hi[a], v[a]); }
+    }
+    __device__ __forceinline__ double mid(int a) const { return 0.5 * (lo[a] + hi[a]); }
+};
+__device__ __forceinline__ double dist2_exact(const double *v, const double *c)
 {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
-    if (i >= n) return;
-    const BvhNode nd = in[i];
-    const int first = nd.left < 0 ? nd.right : nd.pad;
-    float s[3] = {0.f, 0.f, 0.f};
-    for (int k = lane; k < nd.count; k += 32) {
-        const float *v = leaf[first + k].v;
-        const float a[3] = {v[3] - v[0], v[4] - v[1], v[5] - v[2]}, b[3] = {v[6] - v[0], v[7] - v[1], v[8] - v[2]};
-        s[0] += a[1] * b[2] - a[2] * b[1];
-        s[1] += a[2] * b[0] - a[0] * b[2];
-        s[2] += a[0] * b[1] - a[1] * b[0];
-    }
-    for (int o = 16; o > 0; o >>= 1)
-        for (int a = 0; a < 3; ++a) s[a] += __shfl_xor_sync(0xFFFFFFFFu, s[a], o);
-    const float q = sqrtf(fmaf(s[0], s[0], fmaf(s[1], s[1], s[2] * s[2])));
-    const bool flat = q > 0.f && q < INFINITY;
-    float nrm[3] = {flat ? s[0] / q : 1.f, flat ? s[1] / q : 0.f, flat ? s[2] / q : 0.f};
-    float lo = INFINITY, hi = -INFINITY, far = 0.f;
-    for (int k = lane; k < nd.count; k += 32) {
-        const float *v = leaf[first + k].v;
-        for (int m = 0; m < 3; ++m) {
-            const float d[3] = {v[3 * m] - nd.c[0], v[3 * m + 1] - nd.c[1], v[3 * m + 2] - nd.c[2]};
-            const float h = fmaf(d[0], nrm[0], fmaf(d[1], nrm[1], d[2] * nrm[2]));
-            lo = fminf(lo, h);
-            hi = fmaxf(hi, h);
-            far = fmaxf(far, fmaxf(fabsf(v[3 * m]), fmaxf(fabsf(v[3 * m + 1]), fabsf(v[3 * m + 2]))));
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-        far = fmaxf(far, __shfl_xor_sync(0xFFFFFFFFu, far, o));
-    }
-    if (lane == 0) {
-        const float pad = 1e-6f * (far + nd.rad);   // the rounding of the heights and of the unit length
-        NodeRec r;
-        r.sph = make_float4(nd.c[0], nd.c[1], nd.c[2], nd.rad);
-        r.left = nd.left;
-        r.first = first;
-        r.count = nd.left < 0 ? nd.count : 0;
-        r.hi = hi + pad;
-        r.n_lo = make_float4(nrm[0], nrm[1], nrm[2], lo - pad);
-        out[i] = r;
-    }
+    const double dx = v[0] - c[0], dy = v[1] - c[1], dz = v[2] - c[2];
+    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+__device__ __forceinline__ float padded_radius(double d2)
+{
+    return (float)__dadd_rn(__dmul_rn(sqrt(d2), 1.0 + 1e-6), 1e-6);
 }
 
-cudaError_t launch_node_records(int n, const BvhNode *in, const LeafRec *leaf, NodeRec *out, cudaStream_t st)
-{
-    k_node_records<<<(n + 3) / 4, 128, 0, st>>>(n, in, leaf, out);
-    return cudaGetLastError();
-}
-
-__global__ void k_leaf_records(int n, const float *Vf, const int32_t *T, const float *tri_sphere,
-                               const int32_t *tri_order, LeafRec *out)
+__global__ void k_leaf_records(int n, const double *V, const int32_t *T, const int32_t *order, LeafRec *out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int t = tri_order[i];
+    const int t = order[i];
     LeafRec r;
-    r.sph = make_float4(tri_sphere[4 * t], tri_sphere[4 * t + 1], tri_sphere[4 * t + 2], tri_sphere[4 * t + 3]);
-    for (int m = 0; m < 3; ++m)
-        for (int a = 0; a < 3; ++a) r.v[3 * m + a] = Vf[3 * (size_t)T[3 * t + m] + a];
+    BoxD box;
+    const double *v[3];
+    for (int m = 0; m < 3; ++m) {
+        v[m] = V + 3 * (size_t)T[3 * t + m];
+        box.add(v[m]);
+        for (int a = 0; a < 3; ++a) r.v[3 * m + a] = (float)v[m][a];
+    }
+    const double c[3] = {box.mid(0), box.mid(1), box.mid(2)};
+    double d2 = 0.0;
+    for (int m = 0; m < 3; ++m) d2 = fmax(d2, dist2_exact(v[m], c));
+    r.sph = make_float4((float)c[0], (float)c[1], (float)c[2], padded_radius(d2));
     r.tri = t;
     r.pad[0] = r.pad[1] = 0.f;
     out[i] = r;
 }
 
-cudaError_t launch_leaf_records(int n, const float *Vf, const int32_t *T, const float *tri_sphere,
-                                const int32_t *tri_order, LeafRec *out, cudaStream_t st)
+cudaError_t launch_leaf_records(int n, const double *V, const int32_t *T, const int32_t *order, LeafRec *out,
+                                cudaStream_t st)
 {
-    k_leaf_records<<<(n + 127) / 128, 128, 0, st>>>(n, Vf, T, tri_sphere, tri_order, out);
+    k_leaf_records<<<(n + 127) / 128, 128, 0, st>>>(n, V, T, order, out);
+    return cudaGetLastError();
+}
+
+// The value all threads of the group (a warp, or a block of NT threads) agree on.
+template <int NT, class X, class Op> __device__ __forceinline__ X group_all(X x, Op op, X *buf)
+{
+    for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(0xFFFFFFFFu, x, o));
+    if (NT > 32) {
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) buf[threadIdx.x / 32] = x;
+        __syncthreads();
+        x = buf[0];
+        for (int k = 1; k < NT / 32; ++k) x = op(x, buf[k]);
+    }
+    return x;
+}
+
+// NT threads per node (32: a warp, four nodes a block; 1024: a block, for the
+// few nodes of thousands of triangles) over its triangles: box and sphere from
+// the FP64 vertices, then the slab along the area-weighted normal.
+template <int NT>
+__global__ void __launch_bounds__(NT == 32 ? 128 : NT)
+k_node_records(int n, const int32_t *which, const BvhNode *in, const double *V, const int32_t *T, const int32_t *order,
+               const LeafRec *leaf, NodeRec *out)
+{
+    __shared__ double buf[NT == 32 ? 1 : NT / 32];
+    const int g = NT == 32 ? (blockIdx.x * blockDim.x + threadIdx.x) / 32 : blockIdx.x, lane = threadIdx.x % NT;
+    if (g >= n) return;
+    const int i = which ? which[g] : g;
+    const BvhNode nd = in[i];
+    auto mn = [](double a, double b) { return fmin(a, b); };
+    auto mx = [](double a, double b) { return fmax(a, b); };
+    auto sum = [](double a, double b) { return a + b; };
+    BoxD box;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int k = lane; k < nd.count; k += NT) {
+        const int t = order[nd.first + k];
+        for (int m = 0; m < 3; ++m) box.add(V + 3 * (size_t)T[3 * t + m]);
+        const float *v = leaf[nd.first + k].v;
+        const float a[3] = {v[3] - v[0], v[4] - v[1], v[5] - v[2]}, b[3] = {v[6] - v[0], v[7] - v[1], v[8] - v[2]};
+        s[0] += (double)(a[1] * b[2] - a[2] * b[1]);
+        s[1] += (double)(a[2] * b[0] - a[0] * b[2]);
+        s[2] += (double)(a[0] * b[1] - a[1] * b[0]);
+    }
+    double c[3];
+    for (int a = 0; a < 3; ++a) {
+        box.lo[a] = group_all<NT>(box.lo[a], mn, buf);
+        box.hi[a] = group_all<NT>(box.hi[a], mx, buf);
+        s[a] = group_all<NT>(s[a], sum, buf);
+        c[a] = box.mid(a);
+    }
+    const double q = sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
+    const bool flat = q > 0.0 && q < 1e300;
+    const float nrm[3] = {flat ? (float)(s[0] / q) : 1.f, flat ? (float)(s[1] / q) : 0.f, flat ? (float)(s[2] / q) : 0.f};
+    const float cf[3] = {(float)c[0], (float)c[1], (float)c[2]};
+    double d2 = 0.0, lo = 1e300, hi = -1e300, far = 0.0;
+    for (int k = lane; k < nd.count; k += NT) {
+        const int t = order[nd.first + k];
+        const float *vf = leaf[nd.first + k].v;
+        for (int m = 0; m < 3; ++m) {
+            d2 = fmax(d2, dist2_exact(V + 3 * (size_t)T[3 * t + m], c));
+            const float d[3] = {vf[3 * m] - cf[0], vf[3 * m + 1] - cf[1], vf[3 * m + 2] - cf[2]};
+            const double h = (double)fmaf(d[0], nrm[0], fmaf(d[1], nrm[1], d[2] * nrm[2]));
+            lo = fmin(lo, h);
+            hi = fmax(hi, h);
+            far = fmax(far, (double)fmaxf(fabsf(vf[3 * m]), fmaxf(fabsf(vf[3 * m + 1]), fabsf(vf[3 * m + 2]))));
+        }
+    }
+    d2 = group_all<NT>(d2, mx, buf);
+    lo = group_all<NT>(lo, mn, buf);
+    hi = group_all<NT>(hi, mx, buf);
+    far = group_all<NT>(far, mx, buf);
+    if (lane == 0) {
+        NodeRec r;
+        const float rad = padded_radius(d2);
+        const float pad = 1e-6f * ((float)far + rad);   // the rounding of the heights and of the unit length
+        r.sph = make_float4(cf[0], cf[1], cf[2], rad);
+        r.left = nd.left;
+        r.first = nd.first;
+        r.count = nd.left < 0 ? nd.count : 0;
+        r.hi = (float)hi + pad;
+        r.n_lo = make_float4(nrm[0], nrm[1], nrm[2], (float)lo - pad);
+        out[i] = r;
+    }
+}
+
+cudaError_t launch_node_records(int n, int n_big, const int32_t *big, const BvhNode *in, const double *V,
+                                const int32_t *T, const int32_t *order, const LeafRec *leaf, NodeRec *out,
+                                cudaStream_t st)
+{
+    if (n_big > 0)
+        k_node_records<1024><<<n_big, 1024, 0, st>>>(n_big, big, in, V, T, order, leaf, out);
+    k_node_records<32><<<(n - n_big + 3) / 4, 128, 0, st>>>(n - n_big, big + n_big, in, V, T, order, leaf, out);
     return cudaGetLastError();
 }
 
