@@ -305,20 +305,21 @@ __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, 
 //
 // A warp takes 32 consecutive poses (one per lane; consecutive poses of a
 // trajectory are nearly identical) and walks the rows their cylinders reach
-// in lockstep.  On a row each lane estimates its pose's interval in FP32
-// (measured from the point of the row nearest the probe axis, so the estimate
-// carries no cancellation) and proposes the voxels at least CORE_M inside it
-// as its core; the core's two end voxels are classified exactly, and since the
-// cylinder is convex both inside means the whole core is inside.  If the cores
-// of all such lanes share a voxel, every lane's exact interval contains it, so
-// the union of the lanes' intervals is one interval: the warp sets its known
-// part [min core start, max core end] and extends it outward one voxel at a
-// time, asking every lane to classify the voxel, until no lane holds it.
-// Voxels already set in the slab are stepped over unclassified (they are in
-// the result whatever this warp decides, and the union being an interval
-// keeps the stop rule valid).  Lanes whose estimate is unusable (axis nearly
-// along the row, short intervals, failed core ends, or cores that do not
-// overlap) classify their row voxel by voxel with vox_row.
+// in lockstep.  On a row each lane brackets its pose's interval in FP32: an
+// outer interval that holds every voxel of the cylinder and an inner one whose
+// voxels are all inside, apart by the error bound of the coordinates.  Along the
+// rows of a slab the point of the row nearest the probe axis, its distance from
+// the axis and the cap crossings are linear in jy, so a row costs one FMA for
+// each and two square roots.  The union of the inner intervals is one interval
+// when they overlap (the usual case); voxels that some lane's outer interval
+// holds beyond that union and that are not set yet are classified one by one,
+// the exact FP64 predicate deciding inside the error band: only the lanes at the
+// ends of the union can have any.  Lanes whose axis is nearly along the row
+// classify their row voxel by voxel with vox_row.
+//
+// Bound by instruction issue: at N = 128 and 5000 poses a rotation walked 144 000
+// rows of 270 warp instructions when every lane settled its own two ends (44.0 us
+// a rotation, now 18.3; 6.2 -> 3.5 us at N = 64 and 2000 poses).
 template <int N>
 __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *poses, int P, int jz, uint32_t *bits,
                               int *next_chunk)
@@ -332,11 +333,12 @@ __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *pos
     const double h = g.h, r2d = g.r * g.r, Ld = g.L;
     const float ih = g.inv_h;
     const float *Rf = rr.Rf;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
     const float fz = (float)jz;
+    // slack of the row range (voxels): far above the error of the coordinates,
+    // of sqrt(1 - A^2) near 1 (5e-4) times the radius, and of positions along a long probe
+    const float slack = 0.05f + 2e-3f * rv + 1e-5f * lv;
     const volatile uint32_t *vb = bits;
-    (void)warp;
-    (void)nwarp;
     for (;;) {
         // warps take chunks of 32 poses from a block-wide counter, so a warp
         // that drew chunks far from this slab goes on to the next chunk
@@ -352,7 +354,7 @@ __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *pos
             const PoseRec &pr = poses[i];
             float cz = (fmaf(Rf[2], pr.tf[0], fmaf(Rf[5], pr.tf[1], Rf[8] * pr.tf[2])) - rr.of[2]) * ih;
             float Az = fmaf(Rf[2], pr.Rf[2], fmaf(Rf[5], pr.Rf[5], Rf[8] * pr.Rf[8]));
-            float sz = rv * sqrtf(fmaxf(0.f, 1.f - Az * Az)) + 1.5f;
+            float sz = rv * sqrtf(fmaxf(0.f, 1.f - Az * Az)) + slack;
             float z0 = fminf(cz, cz + lv * Az) - sz, z1 = fmaxf(cz, cz + lv * Az) + sz;
             if (!(fz < z0 || fz > z1)) {
                 pose_frame(rr, pr, ih, B, c);
@@ -367,7 +369,7 @@ __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *pos
                     u1 = lv;
                 }
                 if (u0 <= u1) {
-                    float sy = rv * sqrtf(fmaxf(0.f, 1.f - Ay * Ay)) + 1.5f;
+                    float sy = rv * sqrtf(fmaxf(0.f, 1.f - Ay * Ay)) + slack;
                     float ylo = c[1] + fminf(u0 * Ay, u1 * Ay) - sy, yhi = c[1] + fmaxf(u0 * Ay, u1 * Ay) + sy;
                     y0 = max(0, (int)ceilf(ylo));
                     y1 = min(N - 1, (int)floorf(yhi));
@@ -383,122 +385,93 @@ __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *pos
         // per-pose constants of the row walk: the row direction in the probe frame
         const float Aq = fmaf(bx[0], bx[0], bx[1] * bx[1]);
         const bool radial_ok = Aq >= 0.05f;          // axis not within ~13 deg of the row direction
-        const float iAq = radial_ok ? 1.f / Aq : 0.f;
-        const bool cap_ok = fabsf(bx[2]) >= 1e-3f;     // cap crossings located to < 0.25 voxel
-        const float ibz = cap_ok ? 1.f / bx[2] : 0.f;
-        const float rsAq = radial_ok ? rsqrtf(Aq) : 0.f;
-        const float ez = cap_ok ? ELB * fabsf(ibz) : 0.f;   // cap crossings: error of l2 / |bz|
-        const float erq = ELB * rv * iAq;
-        // l0(jy) = B^T ((0, jy, jz) - c) = B_y^T jy + base: one FMA per coordinate per row
+        const float iAq = radial_ok ? 1.f / Aq : 0.f, rsAq = radial_ok ? rsqrtf(Aq) : 0.f;
+        const bool cap_ok = fabsf(bx[2]) >= 1e-3f;
+        // l0(jy) = B^T ((0, jy, jz) - c) = B_y jy + lbase
         float lbase[3];
         for (int k = 0; k < 3; ++k) lbase[k] = fmaf(B[0 * 3 + k], -c[0], fmaf(B[1 * 3 + k], -c[1], B[2 * 3 + k] * (fz - c[2])));
+        // nearest point of the row to the axis: js = js0 + djs jy; signed distance of the row from the axis: d0 + dd jy
+        const float js0 = -fmaf(lbase[0], bx[0], lbase[1] * bx[1]) * iAq, djs = -fmaf(B[3], bx[0], B[4] * bx[1]) * iAq;
+        const float d0 = fmaf(lbase[0], bx[1], -lbase[1] * bx[0]) * rsAq, dd = fmaf(B[3], bx[1], -B[4] * bx[0]) * rsAq;
+        // cap crossings: the nearer one zn0 + dzn jy, the farther zlen on.  Without a usable crossing (the
+        // row nearly parallel to the caps: z moves < N/1000 voxels along it) the row is asked for its z range.
+        const float ibz = cap_ok ? 1.f / bx[2] : 0.f;
+        const float zlen = cap_ok ? lv * fabsf(ibz) : 0.f;
+        const float zn0 = cap_ok ? fmaf(-lbase[2], ibz, bx[2] > 0.f ? 0.f : lv * ibz) : 0.f, dzn = cap_ok ? -B[5] * ibz : 0.f;
+        // error of the chord's middle and ends (rounding included), and of the cap crossings
+        const float e2 = fmaf(ELB, rsAq, 1e-5f * (fabsf(js0) + (float)N * fabsf(djs) + rv * rsAq));
+        const float ez = fmaf(ELB, fabsf(ibz), 1e-5f * (float)N);
+#pragma unroll 1
         for (int jy = Y0; jy <= Y1; ++jy) {
-            const bool act = hit && jy >= y0 && jy <= y1;
-            int st = 0;            // 0: nothing, 1: exact interval [ia, ib], 2: walk voxel by voxel, 3: few candidates
-            int ia = N, ib = -1;
-            int qa = 0, qb = -1;   // st 3: the candidate voxels
-            float l0[3];
-            if (act) {
-                for (int k = 0; k < 3; ++k) l0[k] = fmaf(B[1 * 3 + k], (float)jy, lbase[k]);
-                if (!radial_ok) {
-                    st = 2;
-                } else {
-                    // nearest point of the row to the axis, then the radial chord around it
-                    const float js = -fmaf(l0[0], bx[0], l0[1] * bx[1]) * iAq;
-                    const float sa = fmaf(js, bx[0], l0[0]), sb = fmaf(js, bx[1], l0[1]);
-                    const float Cs = fmaf(sa, sa, sb * sb) - rv2;
-                    const float disc = -Aq * Cs;
-                    if (disc > 0.f) {
-                        // (the rounding of an approximate square root and
-                        // reciprocal, a few ulp, is far inside the 1e-5
-                        // relative term added to E below)
-                        const float hw = disc * rsqrtf(disc) * iAq;
-                        float lo = js - hw, hi = js + hw;
-                        // error of the chord ends: a radius error dl moves a crossing
-                        // by about dl rv / (Aq hw), the nearest point by dl / sqrt(Aq)
-                        float E = fmaf(erq, __frcp_rn(hw), ELB * rsAq);
-                        bool empty = false, unsure = false;
-                        if (cap_ok) {
-                            const float za = -l0[2] * ibz, zb = (lv - l0[2]) * ibz;
-                            lo = fmaxf(lo, fminf(za, zb));
-                            hi = fminf(hi, fmaxf(za, zb));
-                            E = fmaxf(E, ez);
-                        } else {
-                            // row nearly parallel to the cap planes: z moves < N/1000 voxels along it
-                            const float zA = l0[2], zB = fmaf((float)(N - 1), bx[2], l0[2]);
-                            const float zmin = fminf(zA, zB), zmax = fmaxf(zA, zB);
-                            if (zmax < -0.3f || zmin > lv + 0.3f) empty = true;
-                            else if (!(zmin >= 0.3f && zmax <= lv - 0.3f)) unsure = true;
-                        }
-                        E += 1e-5f * fmaxf(fabsf(lo), fabsf(hi));   // rounding of lo, hi themselves
-                        if (empty || lo > (float)N + 1.f || hi < -2.f || lo > hi + 2.f) {
-                            st = 0;
-                        } else if (unsure || E > 0.25f) {
-                            st = 2;
-                        } else if (hi - lo < 2.f * E + 1.f) {
-                            // short chord: its voxels lie in [lo - E, hi + E]
-                            st = 3;
-                            qa = max(0, (int)floorf(fmaxf(lo - E, -1.f)));
-                            qb = min(N - 1, (int)ceilf(fminf(hi + E, (float)N)));
-                        } else {
-                            // voxels below lo - E are outside, those in (lo + E, hi - E)
-                            // inside (the cylinder is convex); an integer in either
-                            // band is classified exactly
-                            st = 1;
-                            int ka = (int)ceilf(lo - E), kb = (int)floorf(hi + E);
-                            ia = ka;
-                            if ((float)ka <= lo + E && ka >= 0 && ka < N &&
-                                !classify(l0, bx, ka, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz))
-                                ia = ka + 1;
-                            ib = kb;
-                            if ((float)kb >= hi - E && kb >= 0 && kb < N &&
-                                !classify(l0, bx, kb, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz))
-                                ib = kb - 1;
-                            ia = max(ia, 0);
-                            ib = min(ib, N - 1);
-                            if (ia > ib) st = 0;
-                        }
-                    } else if (disc > -1e-2f * (1.f + fabsf(Aq * rv2))) {
-                        // tangent row: the exact chord (if any) is within a quarter
-                        // voxel of js
-                        st = 3;
-                        qa = max(0, (int)floorf(fmaxf(js, -2.f)) - 1);
-                        qb = min(N - 1, (int)ceilf(fminf(js, (float)N + 1.f)) + 1);
-                    }
-                }
+            const float fy = (float)jy;
+            bool act = hit && jy >= y0 && jy <= y1;
+            const float js = fmaf(fy, djs, js0), ds = fmaf(fy, dd, d0);
+            const float disc = fmaf(-ds, ds, rv2);
+            // half lengths of the chord at a radius a little larger and a little smaller
+            const float qo = disc + mr, qi = disc - mr;
+            act = act && (qo > 0.f || !radial_ok);
+            const float ho = fmaf(qo * rsqrtf(fmaxf(qo, 1e-30f)), rsAq, e2);
+            const float hi = fmaf(qi * rsqrtf(fmaxf(qi, 1e-30f)), rsAq, -e2);
+            float lo_o = js - ho, hi_o = js + ho, lo_i = js - hi, hi_i = js + hi;
+            bool inner = qi > 0.f;
+            if (cap_ok) {
+                const float zn = fmaf(fy, dzn, zn0), zf = zn + zlen;
+                lo_o = fmaxf(lo_o, zn - ez);
+                hi_o = fminf(hi_o, zf + ez);
+                lo_i = fmaxf(lo_i, zn + ez);
+                hi_i = fminf(hi_i, zf - ez);
+            } else {
+                const float zA = fmaf(B[5], fy, lbase[2]), zB = fmaf((float)(N - 1), bx[2], zA);
+                const float zmin = fminf(zA, zB), zmax = fmaxf(zA, zB);
+                act = act && !(zmax < -slack || zmin > lv + slack);
+                inner = inner && zmin >= slack && zmax <= lv - slack;
             }
-            // exact intervals: one union when they overlap (the usual case for
-            // consecutive poses), else each lane sets its own
-            if (__any_sync(0xFFFFFFFFu, st == 1)) {
-                const int A = __reduce_min_sync(0xFFFFFFFFu, st == 1 ? ia : N);
-                const int Bm = __reduce_max_sync(0xFFFFFFFFu, st == 1 ? ib : -1);
-                const int mxa = __reduce_max_sync(0xFFFFFFFFu, st == 1 ? ia : -1);
-                const int mnb = __reduce_min_sync(0xFFFFFFFFu, st == 1 ? ib : N);
+            const bool walk = act && !radial_ok;
+            // outer voxels [ao, bo], inner voxels [ai, bi]
+            const int ao = (int)ceilf(fmaxf(lo_o, 0.f)), bo = (int)floorf(fminf(hi_o, (float)(N - 1)));
+            act = act && radial_ok && ao <= bo;
+            const int ai = (int)ceilf(fmaxf(lo_i, 0.f)), bi = (int)floorf(fminf(hi_i, (float)(N - 1)));
+            inner = inner && act && ai <= bi;
+            int A = N, Bm = -1;
+            bool more = act;   // some outer voxel may lie beyond what the inner intervals set
+            if (__any_sync(0xFFFFFFFFu, inner)) {
+                A = __reduce_min_sync(0xFFFFFFFFu, inner ? ai : N);
+                Bm = __reduce_max_sync(0xFFFFFFFFu, inner ? bi : -1);
+                const int mxa = __reduce_max_sync(0xFFFFFFFFu, inner ? ai : -1);
+                const int mnb = __reduce_min_sync(0xFFFFFFFFu, inner ? bi : N);
                 if (mxa <= mnb + 1) {
                     if (lane < NW) {
-                        const int lo = max(A, 32 * lane) - 32 * lane, hi = min(Bm, 32 * lane + 31) - 32 * lane;
-                        if (lo <= hi) {
-                            const uint32_t m = (hi == 31 ? 0xFFFFFFFFu : ((1u << (hi + 1)) - 1u)) & ~((1u << lo) - 1u);
+                        const int lo = max(A, 32 * lane) - 32 * lane, hw = min(Bm, 32 * lane + 31) - 32 * lane;
+                        if (lo <= hw) {
+                            const uint32_t m = (0xFFFFFFFFu >> (31 - hw)) & (0xFFFFFFFFu << lo);
                             if (m & ~vb[jy * NW + lane]) atomicOr(&bits[jy * NW + lane], m);
                         }
                     }
-                } else if (st == 1) {
-                    set_bits(bits + jy * NW, ia, ib);
+                    more = act && (ao < A || bo > Bm);
+                } else {
+                    if (inner) set_bits(bits + jy * NW, ai, bi);
+                    more = act && (!inner || ao < ai || bo > bi);
                 }
             }
-            // short chords: the lanes classify their few candidate voxels together
-            if (__any_sync(0xFFFFFFFFu, st == 3)) {
-                const int len = (st == 3) ? qb - qa + 1 : 0;
-                const int maxlen = __reduce_max_sync(0xFFFFFFFFu, len);
-                for (int k = 0; k < maxlen; ++k) {
-                    const int j = qa + k;
-                    bool in = false;
-                    if (k < len && !((vb[jy * NW + (j >> 5)] >> (j & 31)) & 1u))
-                        in = classify(l0, bx, j, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz);
-                    if (in) atomicOr(&bits[jy * NW + (j >> 5)], 1u << (j & 31));
+            if (__any_sync(0xFFFFFFFFu, more || walk)) {
+                __syncwarp();
+                if (more) {
+                    float l0[3];
+                    for (int k = 0; k < 3; ++k) l0[k] = fmaf(B[1 * 3 + k], fy, lbase[k]);
+#pragma unroll 1
+                    for (int j = ao; j <= bo; ++j) {
+                        if (inner && j == ai) {
+                            j = bi;   // [ai, bi] is set
+                            continue;
+                        }
+                        if ((vb[jy * NW + (j >> 5)] >> (j & 31)) & 1u) continue;
+                        if (classify(l0, bx, j, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz))
+                            atomicOr(&bits[jy * NW + (j >> 5)], 1u << (j & 31));
+                    }
                 }
+                if (walk) vox_row<N>(B, c, jy, jz, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, bits + jy * NW);
+                __syncwarp();
             }
-            if (st == 2) vox_row<N>(B, c, jy, jz, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, bits + jy * NW);
         }
     }
 }
