@@ -1436,12 +1436,15 @@ static dock_status run_pipeline_rots(dock_ctx *ctx, const Geo &g, const ReqDev *
     if (ro_any &&
         (s = ensure(ctx, (void **)&ctx->ogr, &ctx->ogr_n, (size_t)B * g.N * g.N * g.N, sizeof(float))) != DOCK_OK)
         return s;
-    int chunks = g.M * g.P / 32;
+    // blocks of the z pass along the columns; about 5000 blocks in all keep the
+    // last wave small (at most 912 are resident), 16 rotations a block are enough
+    // to share a spectrum tile
+    const int64_t chunks = (int64_t)g.M * g.P / (g.M == 256 && tc.zpass_cols == 32 ? 32 : 16);
     int k = 0;
     for (size_t b0 = r0; b0 < r1; b0 += B, ++k) {
         int nb = (int)std::min<size_t>(B, r1 - b0);
-        int groups_needed = (2 * 152 + chunks - 1) / chunks;
-        int group = tc.group > 0 ? std::min(tc.group, nb) : std::max(1, nb / groups_needed);
+        const int group = tc.group > 0 ? std::min(tc.group, nb)
+                                       : (int)std::max<int64_t>(1, std::min<int64_t>(std::min(16, nb), chunks * nb / 5000));
         const RotRec *rb = rots + b0;
         const int kb = k & 1;
         uint32_t *bk = ovl ? ctx->bits + kb * bsz : ctx->bits;

@@ -918,77 +918,98 @@ cudaError_t launch_rot_export(const Geo &g, const ReqDev *reqs, const RotRec *ro
 }
 
 // ---------------------------------------------------------------------------
-// K_B: per chunk of 32 columns f = ky P + kx: forward FFT along z (N non-zero
+// K_B: per chunk of 16 columns f = ky P + kx: forward FFT along z (N non-zero
 // inputs), multiply by conj(F(O)) / M^3 (for a rotated object: conjugate the
-// tile, multiply by F(S) / M^3), inverse FFT along z.  The spectrum
-// of the chunk stays in registers across the `group` rotations of the block.
+// tile, multiply by F(S) / M^3), inverse FFT along z.  The spectrum tile of the
+// chunk stays in shared memory across the `group` rotations of the block and is
+// reloaded when the request (object) changes.
 // DUAL (label-aware score): each rotation has a second tile, Y2, the
 // transform of the voxels reached only by non-contact poses; its product
 // with conj(F(min(O, 0))) / M^3 is added before the inverse FFT, so one
 // inverse transform yields the sum of both correlations.  Requests without
 // non-contact poses skip the addition and keep the plain result bit for bit.
+// Bound by the memory traffic of Y and Z and the chain of its exchanges: the
+// inputs come straight from global memory into registers, the next tile's in
+// flight during the current one, and blocks of 16 columns (64 to 256 threads)
+// leave four to eight of them on an SM.  With 32 columns staged by 8-byte
+// cp.async and the second spectrum read again per rotation, a rotation took 0.58,
+// 3.74 us (plain, N = 32, 64) and 30.3 us (DUAL, N = 96); now 0.33, 3.05 and 20.0.
 // ---------------------------------------------------------------------------
+template <int M, bool DUAL, int V = 0> struct ZpassCfg {
+    static constexpr int COLS = M == 256 ? 32 : 16, NT = Plan<M, V>::T * COLS;
+    // exchange buffer, spectrum tile(s), twiddles
+    static constexpr size_t SMEM = sizeof(cf) * ((size_t)M * COLS * (DUAL ? 3 : 2) + M);
+    // resident blocks the registers are allotted for
+    static constexpr int MINB = (Plan<M, V>::E <= 8 ? 1024 : DUAL ? 512 : 768) / NT;
+};
+
 template <int M, bool DUAL, int V = 0>
-__global__ void __launch_bounds__(Plan<M, V>::T * 32)
-k_zpass(int P, int B, int group, const float2 *Y, const float2 *Y2, const RotRec *rots, const ReqDev *reqs, float2 *Z,
-        const float2 *tw_g)
+__global__ void __launch_bounds__(ZpassCfg<M, DUAL, V>::NT, ZpassCfg<M, DUAL, V>::MINB)
+k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__restrict__ Y2, const RotRec *rots,
+        const ReqDev *reqs, float2 *Z, const float2 *tw_g)
 {
-    constexpr int N = M / 2, E = Plan<M, V>::E, COLS = 32;
+    using C = ZpassCfg<M, DUAL, V>;
+    constexpr int N = M / 2, E = Plan<M, V>::E, COLS = C::COLS;
     constexpr int R_LAST = Plan<M, V>::R(Plan<M, V>::S - 1);
     constexpr int TPR = DUAL ? 2 : 1;        // tiles per rotation
+    constexpr int EL = E / 2;                // slots of the lower (non-zero) half
     extern __shared__ __align__(16) unsigned char smem[];
-    cf *xb = reinterpret_cast<cf *>(smem);   // [M][COLS]
-    cf *tw = xb + M * COLS;                  // [M]
-    cf *yt = tw + M;                         // two [N][COLS] tiles of Y (double buffer)
-    for (int i = threadIdx.x; i < M; i += blockDim.x) { float2 w = tw_g[i]; tw[i] = cmake(w.x, w.y); }
-    const int chunk = blockIdx.x;
+    cf *xb = reinterpret_cast<cf *>(smem);   // [M][COLS] exchange
+    cf *spt = xb + M * COLS;                 // [M (kz)][COLS]
+    cf *pent = spt + (DUAL ? M * COLS : 0);  // [M (kz)][COLS]: the second spectrum
+    cf *tw = pent + M * COLS;                // [M]
     const int c = threadIdx.x % COLS, j = threadIdx.x / COLS;
     const size_t plane = (size_t)M * P;
-    const size_t f0 = (size_t)chunk * COLS;
+    const int f0 = blockIdx.x * COLS;
     const int b0 = blockIdx.y * group;
-    const int nb = min(group, B - b0);
-    const int nt = nb * TPR;
-    // spectrum values in input-slot order of the inverse transform: slot
-    // s <-> kz = j + (M/E) s; held in registers across the block's rotations
-    // and reloaded when the request (object) changes
-    cf sp[E];
-    int sp_req = -1;
-    // asynchronous copy of tile t's non-zero z rows of this chunk (coalesced 256-byte rows)
-    auto prefetch = [&](int t) {
-        const float2 *src = (DUAL && (t & 1)) ? Y2 : Y;
-        const float2 *Yb = src + (size_t)(b0 + t / TPR) * N * plane + f0;
-        cf *dst = yt + (t & 1) * N * COLS;
-        for (int e = threadIdx.x; e < N * COLS; e += blockDim.x) cp_async8(&dst[e], &Yb[(size_t)(e / COLS) * plane + e % COLS]);
-        cp_async_commit();
-    };
-    if (nt > 0) prefetch(0);
-    cf w[E];
-    for (int t = 0; t < nt; ++t) {
-        if (t + 1 < nt) {
-            prefetch(t + 1);
-            cp_async_wait_one();
-        } else {
-            cp_async_wait_all();
+    const int nt = min(group, B - b0) * TPR;
+    if (nt <= 0) return;
+    for (int i = threadIdx.x; i < M; i += C::NT) { float2 w = tw_g[i]; tw[i] = cmake(w.x, w.y); }
+    auto load = [&](int t, cf *v) {
+        const float2 *src = ((DUAL && (t & 1)) ? Y2 : Y) + (size_t)(b0 + t / TPR) * N * plane + f0 + c;
+#pragma unroll
+        for (int s = 0; s < EL; ++s) {
+            const float2 a = __ldcs(&src[(size_t)in_index<M, V>(j, s) * plane]);   // z < N
+            v[s] = cmake(a.x, a.y);
         }
-        __syncthreads();
-        const int bi = t / TPR;
+    };
+    cf nx[EL];
+    load(0, nx);
+    int sp_req = -1;
+    cf w[E];
+    __syncthreads();   // the twiddles
+#pragma unroll 1
+    for (int t = 0; t < nt; ++t) {
+        cf v[E];
+        // (slots s < E / 2 of the first stage read z < N, the others the padding)
+        static_assert(slot_in_lower_half<M, V>(EL - 1) && !slot_in_lower_half<M, V>(EL), "input slots");
+#pragma unroll
+        for (int s = 0; s < EL; ++s) v[s] = nx[s];
+#pragma unroll
+        for (int s = EL; s < E; ++s) v[s] = cmake(0.f, 0.f);
+        if (t + 1 < nt) load(t + 1, nx);
         const bool second = DUAL && (t & 1);
-        const int req = rots[b0 + bi].req;
-        if (!second && req != sp_req) {
-            const float2 *spec = reqs[req].spec;
+        const int bi = t / TPR, req = rots[b0 + bi].req;
+        if (!second && req != sp_req) {   // block-uniform; each thread reads the entries it writes
+            // tiled spectrum: ((f / 32) M + kz) 32 + f mod 32
+            const size_t at = (size_t)(f0 / 32) * M * 32 + (f0 & 31) + c;
+            const float2 *spec = reqs[req].spec + at;
 #pragma unroll
             for (int s = 0; s < E; ++s) {
-                float2 v = spec[((size_t)chunk * M + (j + (M / E) * s)) * COLS + c];
-                sp[s] = cmake(v.x, v.y);
+                const int kz = j + (M / E) * s;
+                const float2 a = __ldg(&spec[(size_t)kz * 32]);
+                spt[kz * COLS + c] = cmake(a.x, a.y);
+            }
+            if (DUAL && reqs[req].P_nc > 0) {
+                const float2 *pen = reqs[req].spec_pen + at;
+#pragma unroll
+                for (int s = 0; s < E; ++s) {
+                    const int kz = j + (M / E) * s;
+                    const float2 a = __ldg(&pen[(size_t)kz * 32]);
+                    pent[kz * COLS + c] = cmake(a.x, a.y);
+                }
             }
             sp_req = req;
-        }
-        const cf *src = yt + (t & 1) * N * COLS;
-        cf v[E];
-#pragma unroll
-        for (int s = 0; s < E; ++s) {
-            int z = in_index<M, V>(j, s);
-            v[s] = slot_in_lower_half<M, V>(s) ? src[z * COLS + c] : cmake(0.f, 0.f);   // z < N
         }
         fft_column<M, false, 1, V>(v, j, xb, c, COLS, tw);
         // forward output slot (bb, r) holds kz = j + (M/E)(bb + (E/R_LAST) r)
@@ -1000,56 +1021,52 @@ k_zpass(int P, int B, int group, const float2 *Y, const float2 *Y2, const RotRec
             for (int bb = 0; bb < E / R_LAST; ++bb)
 #pragma unroll
                 for (int r = 0; r < R_LAST; ++r) {
-                    int k = bb + (E / R_LAST) * r;
+                    const int k = bb + (E / R_LAST) * r;
                     cf a = v[bb * R_LAST + r];
                     a.y *= cj;
-                    w[k] = cmul(a, sp[k]);
+                    w[k] = cmul(a, spt[(j + (M / E) * k) * COLS + c]);
                 }
         } else if (reqs[req].P_nc > 0) {
-            const float2 *pen = reqs[req].spec_pen;
 #pragma unroll
             for (int bb = 0; bb < E / R_LAST; ++bb)
 #pragma unroll
                 for (int r = 0; r < R_LAST; ++r) {
-                    int k = bb + (E / R_LAST) * r;
-                    float2 q = pen[((size_t)chunk * M + (j + (M / E) * k)) * COLS + c];
-                    w[k] = cadd(w[k], cmul(v[bb * R_LAST + r], cmake(q.x, q.y)));
+                    const int k = bb + (E / R_LAST) * r;
+                    // (written out: how the product is contracted into the sum decides its last bit)
+                    const cf a = v[bb * R_LAST + r], q = pent[(j + (M / E) * k) * COLS + c];
+                    w[k].x = __fadd_rn(w[k].x, __fmaf_rn(a.x, q.x, -__fmul_rn(a.y, q.y)));
+                    w[k].y = __fadd_rn(w[k].y, __fmaf_rn(a.x, q.y, __fmul_rn(a.y, q.x)));
                 }
         }
         if (!DUAL || second) {
-            __syncthreads();
             fft_column<M, true, 1, V>(w, j, xb, c, COLS, tw);
             float2 *Zb = Z + (size_t)(b0 + bi) * M * plane + f0 + c;
 #pragma unroll
-            for (int s = 0; s < E; ++s) {
-                int z = out_index<M, V>(j, s);
-                Zb[(size_t)z * plane] = make_float2(w[s].x, w[s].y);
-            }
+            for (int s = 0; s < E; ++s)
+                __stcs(&Zb[(size_t)out_index<M, V>(j, s) * plane], make_float2(w[s].x, w[s].y));
         }
-        __syncthreads();
     }
 }
 
 template <int MM, bool DUAL, int V = 0>
-static cudaError_t launch_zpass_t(const Geo &g, dim3 grid, int B, int group, const float2 *Y, const float2 *Y2,
+static cudaError_t launch_zpass_t(const Geo &g, int B, int group, const float2 *Y, const float2 *Y2,
                                   const RotRec *rots, const ReqDev *reqs, float2 *Z, const float2 *tw, cudaStream_t st)
 {
-    size_t sm = sizeof(cf) * ((size_t)MM * 32 + MM + (size_t)MM * 32);
-    cudaError_t e = cudaFuncSetAttribute(k_zpass<MM, DUAL, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    using C = ZpassCfg<MM, DUAL, V>;
+    cudaError_t e = cudaFuncSetAttribute(k_zpass<MM, DUAL, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
-    k_zpass<MM, DUAL, V><<<grid, Plan<MM, V>::T * 32, sm, st>>>(g.P, B, group, Y, Y2, rots, reqs, Z, tw);
+    const dim3 grid(g.M * g.P / C::COLS, (B + group - 1) / group);
+    k_zpass<MM, DUAL, V><<<grid, C::NT, C::SMEM, st>>>(g.P, B, group, Y, Y2, rots, reqs, Z, tw);
     return cudaGetLastError();
 }
 
 cudaError_t launch_zpass(const Geo &g, int B, int group, const float2 *Y, const RotRec *rots, const ReqDev *reqs,
                          float2 *Z, const float2 *tw, cudaStream_t st, const float2 *Y2, int fft_plan)
 {
-    int chunks = g.M * g.P / 32;
-    dim3 grid(chunks, (B + group - 1) / group);
     switch (g.M) {
 #define ZCASE(MM, V)                                                                                 \
-        return Y2 ? launch_zpass_t<MM, true, V>(g, grid, B, group, Y, Y2, rots, reqs, Z, tw, st)     \
-                  : launch_zpass_t<MM, false, V>(g, grid, B, group, Y, nullptr, rots, reqs, Z, tw, st);
+        return Y2 ? launch_zpass_t<MM, true, V>(g, B, group, Y, Y2, rots, reqs, Z, tw, st)           \
+                  : launch_zpass_t<MM, false, V>(g, B, group, Y, nullptr, rots, reqs, Z, tw, st);
     case 64:
         if (fft_plan == 1) ZCASE(64, 1)
         ZCASE(64, 0)
@@ -1064,37 +1081,296 @@ cudaError_t launch_zpass(const Geo &g, int B, int group, const float2 *Y, const 
 }
 
 // ---------------------------------------------------------------------------
-// K_C: plane z of rotation b: inverse FFT along y of every packed column
-// (column 0 carries kx = 0 + i kx = M/2), then C2R along x of every row by a
-// half-length complex inverse FFT, and the argmax with the lowest linear
-// index on ties.  For M = 256 the plane (256 KB) is split over a 2-CTA
-// cluster; each CTA reads the other half of its rows through distributed
-// shared memory.
+// K_C for M = 64, 128, 192: plane z of rotation b in one CTA: inverse FFT along y
+// of every packed column (column 0 carries kx = 0 + i kx = M/2), then C2R along
+// x of every row by a half-length complex inverse FFT, and the argmax with the
+// lowest linear index on ties.
+//
+// The plane lives in the CTA's registers: a thread holds RA columns' share in
+// phase 1 and RB rows' share in phase 2, and the stages exchange in place through
+// one [M][H + 1] buffer (odd pitch: a warp's 32 rows of one column and its 32
+// columns of one row both hit distinct banks).  Five to nine block barriers a
+// plane (two per exchange), where rounds of 32 columns and rows through a second
+// buffer took about 24 with half as many warps on an SM: 0.53, 4.35, 21.2 us a
+// rotation at N = 32, 64, 96; now 0.40, 3.29, 16.9.
 // ---------------------------------------------------------------------------
-template <int M, int V = 0> struct PlaneCfg {
-    static constexpr int CL = (M >= 256) ? 2 : 1;          // CTAs per plane
+template <int M, int V = 0> struct PlaneRegCfg {
+    static constexpr int H = M / 2, VH = HasPlan<H, V>::value ? V : 0, PP = H + 1;
+    static constexpr int TA = Plan<M, V>::T, EA = Plan<M, V>::E;    // phase 1: threads and values per column
+    static constexpr int TB = Plan<H, VH>::T, EB = Plan<H, VH>::E;  // phase 2: per row
+    static constexpr int NT = M == 64 ? 256 : M == 128 ? 512 : 768;
+    static constexpr int RA = H * TA / NT < 1 ? 1 : H * TA / NT, RB = M * TB / NT < 1 ? 1 : M * TB / NT;
+    static constexpr int MINB = M == 64 ? 6 : M == 128 ? 2 : 1;     // resident CTAs per SM
+    static constexpr size_t SMEM = sizeof(cf) * ((size_t)M * PP + M);   // plane + twiddles
+};
+
+// One exchange of stage s -> s + 1 of a length-L transform through `buf`, the
+// element stride `es` and offset `at` of this thread's column or row.
+template <int L, int s, int V>
+__device__ __forceinline__ void put_stage(const cf *v, int t, cf *buf, int es)
+{
+    constexpr int R = Plan<L, V>::R(s), E = Plan<L, V>::E, T = Plan<L, V>::T, NS = Ns<L, s, V>::v;
+#pragma unroll
+    for (int b = 0; b < E / R; ++b) {
+        const int j = t + T * b, base = (j / NS) * NS * R + (j % NS);
+#pragma unroll
+        for (int r = 0; r < R; ++r) buf[(base + r * NS) * es] = v[b * R + r];
+    }
+}
+template <int L, int s, int V>
+__device__ __forceinline__ void get_stage(cf *v, int t, const cf *buf, int es)
+{
+    constexpr int R = Plan<L, V>::R(s), E = Plan<L, V>::E, T = Plan<L, V>::T;
+#pragma unroll
+    for (int b = 0; b < E / R; ++b) {
+        const int j = t + T * b;
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[b * R + r] = buf[(j + r * (L / R)) * es];
+    }
+}
+
+template <int M, bool EXPORT, int V = 0>
+__global__ void __launch_bounds__(PlaneRegCfg<M, V>::NT, PlaneRegCfg<M, V>::MINB)
+k_plane_reg(const float2 *__restrict__ Z, const float2 *tw_g, const RotRec *rots, const ReqDev *reqs, float *Cout)
+{
+    using C = PlaneRegCfg<M, V>;
+    constexpr int H = C::H, VH = C::VH, PP = C::PP, P = H + 2, NT = C::NT, RA = C::RA, RB = C::RB, EA = C::EA, EB = C::EB;
+    extern __shared__ __align__(16) unsigned char smem[];
+    cf *pb = reinterpret_cast<cf *>(smem);   // [M][PP]
+    cf *tw = pb + M * PP;                    // [M]
+    const int tid = threadIdx.x, zc = blockIdx.x, b = blockIdx.y;
+    const float2 *Zp = Z + ((size_t)b * M + zc) * ((size_t)M * P);
+
+    // ---- phase 1: column c = tid mod H of round rr, index j (warp-uniform) ----
+    constexpr int JA = NT / H;   // threads of a column per round
+    static_assert(NT % H == 0 && JA * RA >= C::TA && H % 32 == 0, "column mapping");
+    {
+        const int c = tid % H, j0 = tid / H;
+        cf v[RA][EA];
+#pragma unroll
+        for (int rr = 0; rr < RA; ++rr) {
+            const int j = j0 + JA * rr;
+            const bool on = C::TA % JA == 0 || j < C::TA;
+#pragma unroll
+            for (int s = 0; s < EA; ++s) {
+                float2 a = make_float2(0.f, 0.f);
+                if (on) a = __ldcs(&Zp[in_index<M, V>(j, s) * P + c]);
+                v[rr][s] = cmake(a.x, a.y);
+            }
+            if (c == 0 && on) {   // + i Z[ky][M/2]
+#pragma unroll
+                for (int s = 0; s < EA; ++s) {
+                    const float2 u = __ldcs(&Zp[in_index<M, V>(j, s) * P + H]);
+                    v[rr][s] = cmake(v[rr][s].x - u.y, v[rr][s].y + u.x);
+                }
+            }
+        }
+        for (int i = tid; i < M; i += NT) { float2 w = tw_g[i]; tw[i] = cmake(w.x, w.y); }
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < RA; ++rr) {
+            const int j = j0 + JA * rr;
+            if (C::TA % JA == 0 || j < C::TA) {
+                stage_compute<M, 0, true, 1, V>(v[rr], j, tw);
+                put_stage<M, 0, V>(v[rr], j, pb + c, PP);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < RA; ++rr) {
+            const int j = j0 + JA * rr;
+            if (C::TA % JA == 0 || j < C::TA) get_stage<M, 1, V>(v[rr], j, pb + c, PP);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < RA; ++rr) {
+            const int j = j0 + JA * rr;
+            if (C::TA % JA == 0 || j < C::TA) {
+                stage_compute<M, 1, true, 1, V>(v[rr], j, tw);
+                put_stage<M, 1, V>(v[rr], j, pb + c, PP);
+            }
+        }
+        __syncthreads();
+        if constexpr (Plan<M, V>::S >= 3) {
+#pragma unroll
+            for (int rr = 0; rr < RA; ++rr) {
+                const int j = j0 + JA * rr;
+                if (C::TA % JA == 0 || j < C::TA) get_stage<M, 2, V>(v[rr], j, pb + c, PP);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int rr = 0; rr < RA; ++rr) {
+                const int j = j0 + JA * rr;
+                if (C::TA % JA == 0 || j < C::TA) {
+                    stage_compute<M, 2, true, 1, V>(v[rr], j, tw);
+                    put_stage<M, 2, V>(v[rr], j, pb + c, PP);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    // ---- phase 2: C2R along x of row y = tid mod M, index j (warp-uniform) ----
+    constexpr int JB = NT / M;
+    static_assert(NT % M == 0 && JB * RB >= C::TB && M % 32 == 0, "row mapping");
+    const int y = tid % M, j0 = tid / M;
+    cf *row = pb + y * PP;
+    cf v[RB][EB];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+        const int j = j0 + JB * rr;
+        if (C::TB % JB == 0 || j < C::TB) {
+#pragma unroll
+            for (int s = 0; s < EB; ++s) {
+                const int k = in_index<H, VH>(j, s);
+                cf Wk, Wm;   // W[k] and W[H - k]; column 0 holds W[0] + i W[H]
+                if (k == 0) {
+                    const cf p = row[0];
+                    Wk = cmake(p.x, 0.f);
+                    Wm = cmake(p.y, 0.f);
+                } else {
+                    Wk = row[k];
+                    Wm = row[H - k];
+                }
+                const cf wc = cconj(Wm);
+                const cf Ek = cadd(Wk, wc);
+                const cf Ok = cmul(csub(Wk, wc), cconj(tw[k]));   // exp(+2 pi i k / M)
+                v[rr][s] = cmake(Ek.x - Ok.y, Ek.y + Ok.x);         // E + i O
+            }
+        }
+    }
+    __syncthreads();   // every W is in registers
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+        const int j = j0 + JB * rr;
+        if (C::TB % JB == 0 || j < C::TB) {
+            stage_compute<H, 0, true, 2, VH>(v[rr], j, tw);
+            put_stage<H, 0, VH>(v[rr], j, row, 1);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+        const int j = j0 + JB * rr;
+        if (C::TB % JB == 0 || j < C::TB) get_stage<H, 1, VH>(v[rr], j, row, 1);
+    }
+    if constexpr (Plan<H, VH>::S >= 3) {
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < RB; ++rr) {
+            const int j = j0 + JB * rr;
+            if (C::TB % JB == 0 || j < C::TB) {
+                stage_compute<H, 1, true, 2, VH>(v[rr], j, tw);
+                put_stage<H, 1, VH>(v[rr], j, row, 1);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < RB; ++rr) {
+            const int j = j0 + JB * rr;
+            if (C::TB % JB == 0 || j < C::TB) get_stage<H, 2, VH>(v[rr], j, row, 1);
+        }
+    }
+    constexpr int LAST = Plan<H, VH>::S - 1;
+    unsigned long long kk = 0ull;
+    const uint32_t rowbase = ((uint32_t)zc * M + (uint32_t)y) * M;
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+        const int j = j0 + JB * rr;
+        if (!(C::TB % JB == 0 || j < C::TB)) continue;
+        stage_compute<H, LAST, true, 2, VH>(v[rr], j, tw);
+        if constexpr (EXPORT) {
+#pragma unroll
+            for (int s = 0; s < EB; ++s) {
+                const uint32_t base = rowbase + 2u * out_index<H, VH>(j, s);
+                Cout[base] = v[rr][s].x;
+                Cout[base + 1] = v[rr][s].y;
+            }
+        } else {
+            // the thread's maximum first; the canvas index (lowest among
+            // equal values) only for the values that reach it
+            float m = v[rr][0].x;
+#pragma unroll
+            for (int s = 0; s < EB; ++s) m = fmaxf(m, fmaxf(v[rr][s].x, v[rr][s].y));
+            if ((uint32_t)(pack_key(m, 0u) >> 32) >= (uint32_t)(kk >> 32)) {
+                uint32_t bi = 0xFFFFFFFFu;
+#pragma unroll
+                for (int s = 0; s < EB; ++s) {
+                    const uint32_t base = rowbase + 2u * out_index<H, VH>(j, s);
+                    if (v[rr][s].x == m) bi = min(bi, base);
+                    if (v[rr][s].y == m) bi = min(bi, base + 1u);
+                }
+                if (bi != 0xFFFFFFFFu) {
+                    const unsigned long long k2 = pack_key(m, bi);
+                    kk = k2 > kk ? k2 : kk;
+                }
+            }
+        }
+    }
+    if constexpr (!EXPORT) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long k2 = __shfl_down_sync(0xFFFFFFFFu, kk, o);
+            kk = k2 > kk ? k2 : kk;
+        }
+        __shared__ unsigned long long wk[NT / 32];
+        if ((tid & 31) == 0) wk[tid >> 5] = kk;
+        __syncthreads();
+        if (tid < 32) {
+            kk = tid < NT / 32 ? wk[tid] : 0ull;
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long k2 = __shfl_down_sync(0xFFFFFFFFu, kk, o);
+                kk = k2 > kk ? k2 : kk;
+            }
+            if (tid == 0 && kk) atomicMax(&reqs[rots[b].req].keys[rots[b].rot], kk);
+        }
+    }
+}
+
+template <int M, int V = 0>
+static cudaError_t launch_plane_reg(int B, const float2 *Z, const float2 *tw, const RotRec *rots, const ReqDev *reqs,
+                                    float *C, cudaStream_t st)
+{
+    using Cf = PlaneRegCfg<M, V>;
+    const auto set = [](const void *f) {
+        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cf::SMEM);
+    };
+    cudaError_t e;
+    if (C) {
+        if ((e = set((const void *)k_plane_reg<M, true, V>)) != cudaSuccess) return e;
+        k_plane_reg<M, true, V><<<dim3(M, 1), Cf::NT, Cf::SMEM, st>>>(Z, tw, nullptr, nullptr, C);
+    } else {
+        if ((e = set((const void *)k_plane_reg<M, false, V>)) != cudaSuccess) return e;
+        k_plane_reg<M, false, V><<<dim3(M, B), Cf::NT, Cf::SMEM, st>>>(Z, tw, rots, reqs, nullptr);
+    }
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// K_C for M = 256 over a 2-CTA cluster per plane (plane_cl = 2, and where the
+// 4- and 8-CTA forms of k_fft256.cu cannot run): the same transforms, the plane
+// (256 KB) split between the CTAs; each reads the other half of its rows through
+// distributed shared memory.
+// ---------------------------------------------------------------------------
+struct PlaneCfg {
+    static constexpr int M = 256, CL = 2;                  // CTAs per plane
     static constexpr int H = M / 2;
-    static constexpr int VH = HasPlan<H, V>::value ? V : 0;   // the C2R's plan (length H)
     static constexpr int PC = H / CL;                      // packed columns per CTA
     static constexpr int PP = PC + 1;                      // odd pitch: a warp's rows hit distinct banks
-    static constexpr int NT = Plan<M, V>::T * 32;             // threads
+    static constexpr int NT = Plan<M>::T * 32;             // threads
     static constexpr int COLS = 32;                        // columns per round of the y transform
-    static constexpr int RPR = NT / Plan<H, VH>::T;            // rows per round of the C2R
+    static constexpr int RPR = NT / Plan<H>::T;            // rows per round of the C2R
     static constexpr int S1 = M * COLS;                    // phase-1 exchange
-    static constexpr int S2 = CL > 1 ? (M / CL) * PP : 0;  // peer rows (cluster only)
-    static constexpr int S3 = H * RPR;                     // phase-2 exchange (single CTA)
-    static constexpr int STG = S1 > S2 ? (S1 > S3 ? S1 : S3) : (S2 > S3 ? S2 : S3);
+    static constexpr int S2 = (M / CL) * PP;               // peer rows
+    static constexpr int STG = S1 > S2 ? S1 : S2;
     static constexpr size_t SMEM = sizeof(cf) * ((size_t)M * PP + STG + 2 * M);   // + twiddles + Nyquist column
     static_assert(SMEM <= 227 * 1024, "plane pass exceeds the shared memory of one CTA");
 };
 
-template <int M, bool EXPORT, int V = 0>
+template <bool EXPORT>
 __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g, unsigned long long *key, float *Cout,
                                            int zc, cf *pb, cf *stg, cf *tw, int rank)
 {
-    using C = PlaneCfg<M, V>;
-    constexpr int VH = C::VH;
-    constexpr int H = M / 2, CL = C::CL, PC = C::PC, PP = C::PP, E = Plan<M, V>::E, COLS = C::COLS;
+    using C = PlaneCfg;
+    constexpr int M = C::M, H = C::H, CL = C::CL, PC = C::PC, PP = C::PP, E = Plan<M>::E, COLS = C::COLS;
     const int P = H + 2;
     for (int i = threadIdx.x; i < M; i += blockDim.x) { float2 w = tw_g[i]; tw[i] = cmake(w.x, w.y); }
     __syncthreads();
@@ -1134,21 +1410,21 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
             const bool act = pl < PC;
             cf v[E];
 #pragma unroll
-            for (int s = 0; s < E; ++s) v[s] = act ? pb[in_index<M, V>(j, s) * PP + pl] : cmake(0.f, 0.f);
-            fft_column<M, true, 1, V>(v, j, stg, c, COLS, tw);
+            for (int s = 0; s < E; ++s) v[s] = act ? pb[in_index<M>(j, s) * PP + pl] : cmake(0.f, 0.f);
+            fft_column<M, true, 1>(v, j, stg, c, COLS, tw);
             if (act) {
 #pragma unroll
-                for (int s = 0; s < E; ++s) pb[out_index<M, V>(j, s) * PP + pl] = v[s];
+                for (int s = 0; s < E; ++s) pb[out_index<M>(j, s) * PP + pl] = v[s];
             }
             __syncthreads();
         }
     }
-    // my rows [rank M/CL, (rank+1) M/CL); with a cluster, the peer's columns of
-    // those rows are copied once (coalesced) into stg, and after a second
-    // barrier the half of pb the peer read is free for the C2R exchange
+    // my rows [rank M/CL, (rank+1) M/CL): the peer's columns of those rows are
+    // copied once (coalesced) into stg, and after a second barrier the half of pb
+    // the peer read is free for the C2R exchange
     const int rows = M / CL, row0 = rank * rows;
-    cf *xb2 = stg;
-    if constexpr (CL > 1) {
+    cf *xb2;
+    {
         cg::cluster_group cl = cg::this_cluster();
         cl.sync();
         const cf *peer = cl.map_shared_rank(pb, rank ^ 1);
@@ -1173,12 +1449,10 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
         }
         cl.sync();
         xb2 = pb + (rank ^ 1) * rows * PP;
-    } else {
-        __syncthreads();
     }
     // phase 2: C2R along x of my rows by a half-length complex inverse FFT
     {
-        constexpr int EH = Plan<H, VH>::E, RPR = C::RPR;
+        constexpr int EH = Plan<H>::E, RPR = C::RPR;
         const int rowl = threadIdx.x % RPR, j = threadIdx.x / RPR;
         float best = -INFINITY;
         uint32_t bidx = 0xFFFFFFFFu;
@@ -1189,14 +1463,14 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
             cf v[EH];
 #pragma unroll
             for (int s = 0; s < EH; ++s) {
-                int k = in_index<H, VH>(j, s);
+                int k = in_index<H>(j, s);
                 cf Ek = cmake(0.f, 0.f), Ok = cmake(0.f, 0.f);
                 if (act) {
                     // W[k] and W[H - k]; column 0 holds W[0] + i W[H]
                     cf Wk, Wm;
                     auto fetch = [&](int col) -> cf {
                         int own = col / PC, l = col % PC;
-                        if (CL == 1 || own == rank) return pb[y * PP + l];
+                        if (own == rank) return pb[y * PP + l];
                         return stg[yl * PP + l];
                     };
                     if (k == 0) {
@@ -1213,13 +1487,13 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
                 }
                 v[s] = cmake(Ek.x - Ok.y, Ek.y + Ok.x);   // E + i O
             }
-            fft_column<H, true, 2, VH>(v, j, xb2, rowl, RPR, tw);
+            fft_column<H, true, 2>(v, j, xb2, rowl, RPR, tw);
             if (act) {
                 const uint32_t rowbase = ((uint32_t)zc * M + (uint32_t)y) * M;
                 if (EXPORT) {
 #pragma unroll
                     for (int s = 0; s < EH; ++s) {
-                        const uint32_t base = rowbase + 2u * out_index<H, VH>(j, s);
+                        const uint32_t base = rowbase + 2u * out_index<H>(j, s);
                         Cout[base] = v[s].x;
                         Cout[base + 1] = v[s].y;
                     }
@@ -1234,7 +1508,7 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
 #pragma unroll
                     for (int s = 0; s < EH; ++s) {
                         if (v[s].x == m || v[s].y == m) {
-                            const uint32_t base = rowbase + 2u * out_index<H, VH>(j, s);
+                            const uint32_t base = rowbase + 2u * out_index<H>(j, s);
                             if (v[s].x == m) bi = min(bi, base);
                             if (v[s].y == m) bi = min(bi, base + 1u);
                         }
@@ -1266,18 +1540,17 @@ __device__ __forceinline__ void plane_body(const float2 *Zp, const float2 *tw_g,
     }
 }
 
-template <int M, int V = 0>
-__global__ void __launch_bounds__(PlaneCfg<M, V>::NT)
+__global__ void __launch_bounds__(PlaneCfg::NT)
 k_plane(int B, const float2 *Z, const float2 *tw_g, const RotRec *rots, const ReqDev *reqs, int ahead)
 {
-    using C = PlaneCfg<M, V>;
+    using C = PlaneCfg;
+    constexpr int M = C::M;
     extern __shared__ __align__(16) unsigned char smem[];
     cf *pb = reinterpret_cast<cf *>(smem);    // [M][PP]
     cf *stg = pb + M * C::PP;                 // [STG]
     cf *tw = stg + C::STG;                    // [M]
     const int zc = blockIdx.x / C::CL, b = blockIdx.y;
-    int rank = 0;
-    if constexpr (C::CL > 1) rank = (int)cg::this_cluster().block_rank();
+    const int rank = (int)cg::this_cluster().block_rank();
     const size_t plane = (size_t)M * (M / 2 + 2);
     const float2 *Zp = Z + ((size_t)b * M + zc) * plane;
     // One CTA fits an SM, so its column loads cannot overlap another CTA's
@@ -1301,37 +1574,33 @@ k_plane(int B, const float2 *Z, const float2 *tw_g, const RotRec *rots, const Re
             asm volatile("prefetch.global.L2 [%0];" ::"l"(row + off));
         }
     }
-    plane_body<M, false, V>(Zp, tw_g, &reqs[rots[b].req].keys[rots[b].rot], nullptr, zc, pb, stg, tw, rank);
+    plane_body<false>(Zp, tw_g, &reqs[rots[b].req].keys[rots[b].rot], nullptr, zc, pb, stg, tw, rank);
 }
 
-template <int M, int V = 0>
-__global__ void __launch_bounds__(PlaneCfg<M, V>::NT)
+__global__ void __launch_bounds__(PlaneCfg::NT)
 k_plane_export(const float2 *Z, const float2 *tw_g, float *C)
 {
-    using Cf = PlaneCfg<M, V>;
+    using Cf = PlaneCfg;
+    constexpr int M = Cf::M;
     extern __shared__ __align__(16) unsigned char smem[];
     cf *pb = reinterpret_cast<cf *>(smem);
     cf *stg = pb + M * Cf::PP;
     cf *tw = stg + Cf::STG;
     const int zc = blockIdx.x / Cf::CL;
-    int rank = 0;
-    if constexpr (Cf::CL > 1) rank = (int)cg::this_cluster().block_rank();
+    const int rank = (int)cg::this_cluster().block_rank();
     const size_t plane = (size_t)M * (M / 2 + 2);
-    plane_body<M, true, V>(Z + (size_t)zc * plane, tw_g, nullptr, C, zc, pb, stg, tw, rank);
+    plane_body<true>(Z + (size_t)zc * plane, tw_g, nullptr, C, zc, pb, stg, tw, rank);
 }
 
-template <int M, int V = 0>
-static size_t plane_smem() { return PlaneCfg<M, V>::SMEM; }
-
-template <int M, bool EXPORT, int V = 0>
-static cudaError_t launch_plane_t(int B, const float2 *Z, const float2 *tw, const RotRec *rots,
+template <bool EXPORT>
+static cudaError_t launch_plane_2(int B, const float2 *Z, const float2 *tw, const RotRec *rots,
                                   const ReqDev *reqs, float *C, cudaStream_t st)
 {
-    constexpr int CL = PlaneCfg<M, V>::CL;
-    size_t sm = plane_smem<M, V>();
+    constexpr int M = PlaneCfg::M, CL = PlaneCfg::CL;
+    const size_t sm = PlaneCfg::SMEM;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(M * CL, EXPORT ? 1 : B);
-    cfg.blockDim = dim3(PlaneCfg<M, V>::NT);
+    cfg.blockDim = dim3(PlaneCfg::NT);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
@@ -1343,18 +1612,18 @@ static cudaError_t launch_plane_t(int B, const float2 *Z, const float2 *tw, cons
     cfg.numAttrs = 1;
     cudaError_t e;
     if (EXPORT) {
-        e = cudaFuncSetAttribute(k_plane_export<M, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = cudaFuncSetAttribute(k_plane_export, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        e = cudaLaunchKernelEx(&cfg, k_plane_export<M, V>, Z, tw, C);
+        e = cudaLaunchKernelEx(&cfg, k_plane_export, Z, tw, C);
     } else {
-        e = cudaFuncSetAttribute(k_plane<M, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = cudaFuncSetAttribute(k_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         // planes in flight at one CTA per SM: the next CTA on an SM takes
         // roughly the plane this many further on
         int dev = 0, sms = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        e = cudaLaunchKernelEx(&cfg, k_plane<M, V>, B, Z, tw, rots, reqs, sms / CL);
+        e = cudaLaunchKernelEx(&cfg, k_plane, B, Z, tw, rots, reqs, sms / CL);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -1370,13 +1639,13 @@ cudaError_t launch_plane(const Geo &g, int B, const float2 *Z, const float2 *tw,
     if (plane_cl_supported(g.M, plane_cl)) return launch_plane_cl(g, plane_cl, B, Z, tw, rots, reqs, err, st);
     switch (g.M) {
     case 64:
-        return fft_plan == 1 ? launch_plane_t<64, false, 1>(B, Z, tw, rots, reqs, nullptr, st)
-                             : launch_plane_t<64, false>(B, Z, tw, rots, reqs, nullptr, st);
+        return fft_plan == 1 ? launch_plane_reg<64, 1>(B, Z, tw, rots, reqs, nullptr, st)
+                             : launch_plane_reg<64>(B, Z, tw, rots, reqs, nullptr, st);
     case 128:
-        return fft_plan == 1 ? launch_plane_t<128, false, 1>(B, Z, tw, rots, reqs, nullptr, st)
-                             : launch_plane_t<128, false>(B, Z, tw, rots, reqs, nullptr, st);
-    case 192: return launch_plane_t<192, false>(B, Z, tw, rots, reqs, nullptr, st);
-    case 256: return launch_plane_t<256, false>(B, Z, tw, rots, reqs, nullptr, st);
+        return fft_plan == 1 ? launch_plane_reg<128, 1>(B, Z, tw, rots, reqs, nullptr, st)
+                             : launch_plane_reg<128>(B, Z, tw, rots, reqs, nullptr, st);
+    case 192: return launch_plane_reg<192>(B, Z, tw, rots, reqs, nullptr, st);
+    case 256: return launch_plane_2<false>(B, Z, tw, rots, reqs, nullptr, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1391,13 +1660,13 @@ cudaError_t launch_plane_export(const Geo &g, const float2 *Z, const float2 *tw,
     if (plane_cl_supported(g.M, plane_cl)) return launch_plane_cl_export(g, plane_cl, Z, tw, C, err, st);
     switch (g.M) {
     case 64:
-        return fft_plan == 1 ? launch_plane_t<64, true, 1>(1, Z, tw, nullptr, nullptr, C, st)
-                             : launch_plane_t<64, true>(1, Z, tw, nullptr, nullptr, C, st);
+        return fft_plan == 1 ? launch_plane_reg<64, 1>(1, Z, tw, nullptr, nullptr, C, st)
+                             : launch_plane_reg<64>(1, Z, tw, nullptr, nullptr, C, st);
     case 128:
-        return fft_plan == 1 ? launch_plane_t<128, true, 1>(1, Z, tw, nullptr, nullptr, C, st)
-                             : launch_plane_t<128, true>(1, Z, tw, nullptr, nullptr, C, st);
-    case 192: return launch_plane_t<192, true>(1, Z, tw, nullptr, nullptr, C, st);
-    case 256: return launch_plane_t<256, true>(1, Z, tw, nullptr, nullptr, C, st);
+        return fft_plan == 1 ? launch_plane_reg<128, 1>(1, Z, tw, nullptr, nullptr, C, st)
+                             : launch_plane_reg<128>(1, Z, tw, nullptr, nullptr, C, st);
+    case 192: return launch_plane_reg<192>(1, Z, tw, nullptr, nullptr, C, st);
+    case 256: return launch_plane_2<true>(1, Z, tw, nullptr, nullptr, C, st);
     default: return cudaErrorInvalidValue;
     }
 }
