@@ -471,22 +471,27 @@ k_plane_ps(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUt
     cg::this_cluster().sync();
 
     bool fail = false;   // block-uniform: a wait of this CTA ran out
-    int key_b = -1;      // (thread 0) rotation whose plane key waits in s_key[key_par]
-    uint32_t key_par = 0;
+    // the key of the plane's rotation.  Its address is a chain of two memory
+    // latencies (rots -> reqs): looked up while the plane's columns arrive and
+    // kept until the plane's key has left, so that no wait of phase 2 or of the
+    // flush begins with it.
+    unsigned long long *rot_key = nullptr;
+    bool key_waits = false;   // (thread 0) the previous plane's key is in s_key
     // the previous plane's key (every warp has added to it before the barrier
     // that precedes this call) goes to its rotation's key array
-    auto flush_key = [&]() {
-        if (!EXPORT && tid == 0 && key_b >= 0) {
+    auto flush_key = [&](uint32_t key_par) {
+        if (!EXPORT && tid == 0 && key_waits) {
             const unsigned long long kk = s_key[key_par];
-            if (kk) atomicMax(&reqs[rots[key_b].req].keys[rots[key_b].rot], kk);
+            if (kk) atomicMax(rot_key, kk);
             s_key[key_par] = 0ull;
-            key_b = -1;
+            key_waits = false;
         }
     };
     int i = 0;
 #pragma unroll 1
     for (int p = cid; p < n_planes; p += G, ++i) {
         const uint32_t par = (uint32_t)(i & 1);
+        const RotRec rec = rots[p >> 8];
         if (!fail) {
             if (tid == 0) mbar_arrive_expect_tx(v_bar, C::CL * C::BLK_BYTES);
             const bool tma_ok = mbar_wait_bounded(tma_bar, par, C::WAIT_CYCLES);
@@ -513,7 +518,8 @@ k_plane_ps(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUt
                 if (tid == 0 && err) atomicExch(err, DOCK_E_TIMEOUT);
             } else {
                 if (tid == 0) tma_out = -1;
-                flush_key();
+                flush_key(par ^ 1u);
+                if (!EXPORT) rot_key = reqs[rec.req].keys + rec.rot;
 #pragma unroll
                 for (int r = 0; r < 16; ++r) V[(16 * j + r) * CPC + c] = v[r];
                 __syncthreads();
@@ -559,11 +565,11 @@ k_plane_ps(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUt
         // ---- phase 2: C2R along x of my rows, argmax -------------------------
         const int rowl = tid & 31, j = (tid >> 5) & 7, rr = tid >> 8;   // j, rr warp-uniform
         const int ylo = rr * 32 + rowl, y = rank * RPC + ylo;
-        const int b = p >> 8, zc = p & (M - 1);
+        const int zc = p & (M - 1);
         // the rotation's best key so far (from the planes done before; a stale
         // value is only lower): a row whose maximum scores below it cannot
         // hold the rotation's peak and skips the search for its index
-        const uint32_t thr = EXPORT ? 0u : (uint32_t)(__ldcg(&reqs[rots[b].req].keys[rots[b].rot]) >> 32);
+        const uint32_t thr = EXPORT ? 0u : (uint32_t)(__ldcg(rot_key) >> 32);
         // element (kx, local row ylo) of V: source kx / CPC, column
         // (kx mod CPC) ^ (y mod CPC) (RPC is a multiple of CPC)
         auto vat = [&](int kx) -> cf { return V[(kx / CPC) * BLK + ylo * CPC + ((kx % CPC) ^ (ylo & (CPC - 1)))]; };
@@ -641,14 +647,11 @@ k_plane_ps(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUt
             // the plane's key in shared memory; thread 0 sends it on after the
             // next barrier (the next plane's, or the one after the loop)
             if ((tid & 31) == 0 && kk) atomicMax(&s_key[par], kk);
-            if (tid == 0) {
-                key_b = b;
-                key_par = par;
-            }
+            key_waits = true;
         }
     }
     __syncthreads();
-    if (!fail) flush_key();
+    if (!fail) flush_key((uint32_t)(i - 1) & 1u);
     // copies this CTA stopped waiting for: wait (bounded) before its shared
     // memory is released
     if (tid == 0) {
@@ -847,7 +850,9 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
     };
     cf nx[8];
     load(0, nx);
-    int sp_req = -1;
+    // (looked up one rotation ahead: rots -> reqs is a chain of two memory latencies)
+    int sp_req = -1, req = rots[b0].req;
+    float cj = 1.f;
 #pragma unroll 1
     for (int bi = 0; bi < nb; ++bi) {
         cf v[16];
@@ -856,7 +861,7 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
 #pragma unroll
         for (int s = 8; s < 16; ++s) v[s] = cmake(0.f, 0.f);   // z >= N: zero padding
         if (bi + 1 < nb) load(bi + 1, nx);
-        const int req = rots[b0 + bi].req;
+        const int next_req = rots[b0 + min(bi + 1, nb - 1)].req;
         if (req != sp_req) {   // block-uniform
             __syncthreads();   // the previous tile is no longer read
             const float2 *spec = reqs[req].spec;
@@ -867,9 +872,9 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
                 const float2 a = __ldg(&src[(size_t)(j + 16 * r) * 32]);
                 spt[(j + 16 * r) * COLS + c] = cmake(a.x, a.y);
             }
+            cj = reqs[req].rotate_object ? -1.f : 1.f;
             sp_req = req;
         }
-        const float cj = reqs[req].rotate_object ? -1.f : 1.f;
         // forward, stage 0 (inputs z = j + 16 s) -> index 16 j + r
         DFT<16, false>::run(v);
 #pragma unroll
@@ -901,6 +906,7 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
         float2 *dst = Z + (size_t)(b0 + bi) * M * plane + f0 + c;
 #pragma unroll
         for (int r = 0; r < 16; ++r) __stcs(&dst[(size_t)(j + 16 * r) * plane], make_float2(v[r].x, v[r].y));
+        req = next_req;
         __syncthreads();   // the exchange buffer is free for the next rotation
     }
 }
@@ -1282,17 +1288,20 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
     cf nx[8], nx2[8];
     load(Y, 0, nx);
     load(Y2, 0, nx2);
-    int sp_req = -1;
+    int sp_req = -1, req = rots[b0].req;   // looked up one rotation ahead
+    bool pen = false;
+    float cj = 1.f;
 #pragma unroll 1
     for (int bi = 0; bi < nb; ++bi) {
         cf v[16], w[16];
 #pragma unroll
         for (int s = 0; s < 8; ++s) v[s] = nx[s];
         if (bi + 1 < nb) load(Y, bi + 1, nx);
-        const int req = rots[b0 + bi].req;
-        const bool pen = reqs[req].P_nc > 0;
+        const int next_req = rots[b0 + min(bi + 1, nb - 1)].req;
         if (req != sp_req) {   // block-uniform
             __syncthreads();   // the previous tiles are no longer read
+            pen = reqs[req].P_nc > 0;
+            cj = reqs[req].rotate_object ? -1.f : 1.f;
             // tiled spectra: ((f / 32) M + kz) 32 + f mod 32
             const size_t off = (size_t)(f0 / 32) * M * 32 + (f0 & 31) + c;
             const float2 *src = reqs[req].spec + off;
@@ -1311,7 +1320,6 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
             }
             sp_req = req;
         }
-        const float cj = reqs[req].rotate_object ? -1.f : 1.f;
         // contact sweep: w = F(S) conj(F(O)) / M^3 (a rotated object: conj(F(O_R)) F(S) / M^3)
         forward(v);
 #pragma unroll
@@ -1346,6 +1354,7 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
         float2 *dst = Z + (size_t)(b0 + bi) * M * plane + f0 + c;
 #pragma unroll
         for (int r = 0; r < 16; ++r) __stcs(&dst[(size_t)(j + 16 * r) * plane], make_float2(w[r].x, w[r].y));
+        req = next_req;
         __syncthreads();   // the exchange buffer is free for the next rotation
     }
 }

@@ -37,7 +37,6 @@ __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src)
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 // wait until at most n (0..3) of this thread's committed groups are pending
 __device__ __forceinline__ void cp_async_wait_pending(int n)
 {
@@ -975,7 +974,10 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
     };
     cf nx[EL];
     load(0, nx);
-    int sp_req = -1;
+    // the request of a rotation is looked up one rotation ahead: rots -> reqs is
+    // a chain of two memory latencies that a tile would otherwise begin with
+    int sp_req = -1, req = rots[b0].req, P_nc = 0;
+    float cj = 1.f;
     cf w[E];
     __syncthreads();   // the twiddles
 #pragma unroll 1
@@ -989,7 +991,7 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
         for (int s = EL; s < E; ++s) v[s] = cmake(0.f, 0.f);
         if (t + 1 < nt) load(t + 1, nx);
         const bool second = DUAL && (t & 1);
-        const int bi = t / TPR, req = rots[b0 + bi].req;
+        const int bi = t / TPR, next_req = rots[b0 + min(t + 1, nt - 1) / TPR].req;
         if (!second && req != sp_req) {   // block-uniform; each thread reads the entries it writes
             // tiled spectrum: ((f / 32) M + kz) 32 + f mod 32
             const size_t at = (size_t)(f0 / 32) * M * 32 + (f0 & 31) + c;
@@ -1000,7 +1002,11 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
                 const float2 a = __ldg(&spec[(size_t)kz * 32]);
                 spt[kz * COLS + c] = cmake(a.x, a.y);
             }
-            if (DUAL && reqs[req].P_nc > 0) {
+            // a rotated object: this tile is F(O_R) and spec is F(S) / M^3,
+            // so the product is conj(F(O_R)) F(S) / M^3 (Eq. (9) read as Eq. (7))
+            cj = reqs[req].rotate_object ? -1.f : 1.f;
+            P_nc = reqs[req].P_nc;
+            if (DUAL && P_nc > 0) {
                 const float2 *pen = reqs[req].spec_pen + at;
 #pragma unroll
                 for (int s = 0; s < E; ++s) {
@@ -1014,9 +1020,6 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
         fft_column<M, false, 1, V>(v, j, xb, c, COLS, tw);
         // forward output slot (bb, r) holds kz = j + (M/E)(bb + (E/R_LAST) r)
         if (!second) {
-            // a rotated object: this tile is F(O_R) and spec is F(S) / M^3,
-            // so the product is conj(F(O_R)) F(S) / M^3 (Eq. (9) read as Eq. (7))
-            const float cj = reqs[req].rotate_object ? -1.f : 1.f;
 #pragma unroll
             for (int bb = 0; bb < E / R_LAST; ++bb)
 #pragma unroll
@@ -1026,7 +1029,7 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
                     a.y *= cj;
                     w[k] = cmul(a, spt[(j + (M / E) * k) * COLS + c]);
                 }
-        } else if (reqs[req].P_nc > 0) {
+        } else if (P_nc > 0) {
 #pragma unroll
             for (int bb = 0; bb < E / R_LAST; ++bb)
 #pragma unroll
@@ -1045,6 +1048,7 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
             for (int s = 0; s < E; ++s)
                 __stcs(&Zb[(size_t)out_index<M, V>(j, s) * plane], make_float2(w[s].x, w[s].y));
         }
+        req = next_req;
     }
 }
 
