@@ -108,6 +108,11 @@ __device__ __forceinline__ cf twc_inv(int m)
     return cmake(w.x, -w.y);
 }
 
+// the 128-byte line of gmem is fetched towards L2; no register waits for it
+__device__ __forceinline__ void prefetch_l2(const void *gmem)
+{
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(gmem));
+}
 }  // namespace
 
 template <int CL> struct PlaneClCfg {
@@ -816,11 +821,16 @@ k_fwd2d_runs(const uint32_t *__restrict__ bits_g, const uint32_t *__restrict__ m
 // the N = 128 non-zero inputs, times conj(F(O)) / M^3 (for a rotated object:
 // the tile conjugated, times F(S) / M^3), inverse FFT along z.  Thread (c, j)
 // (c = column, j < 16) holds z (or kz) = j + 16 s: the inputs come straight
-// from global memory (the next rotation's already in flight), the forward
+// from global memory (the next rotation's on their way to L2), the forward
 // output is in the inverse's input order, and both transforms exchange
 // between their radix-16 stages through one [256][16] buffer.  The block's
 // spectrum tile [kz][16] sits in shared memory (reloaded when the request
 // changes), the stage twiddles come from the constant bank.
+// Bound by the traffic of Y and Z (102 MB a rotation, 15 us at the copy rate).
+// The next rotation's 128 lines are prefetched to L2 and loaded after the last
+// store: holding them in 16 registers during the transforms made the compiler
+// spill, and a spilled load is waited for at once.  25.7 -> 21.4 us a rotation
+// (4.8 TB/s).
 // ---------------------------------------------------------------------------
 struct Zpass16Cfg {
     static constexpr int M = 256, N = 128, P = 130, NT = 256, COLS = 16;
@@ -848,19 +858,17 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
             v[s] = cmake(a.x, a.y);
         }
     };
-    cf nx[8];
-    load(0, nx);
+    cf v[16];
+    load(0, v);
     // (looked up one rotation ahead: rots -> reqs is a chain of two memory latencies)
     int sp_req = -1, req = rots[b0].req;
     float cj = 1.f;
 #pragma unroll 1
     for (int bi = 0; bi < nb; ++bi) {
-        cf v[16];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) v[s] = nx[s];
 #pragma unroll
         for (int s = 8; s < 16; ++s) v[s] = cmake(0.f, 0.f);   // z >= N: zero padding
-        if (bi + 1 < nb) load(bi + 1, nx);
+        // the next rotation's 128 lines of 16 columns, towards L2
+        if (bi + 1 < nb && tid < N) prefetch_l2(Y + ((size_t)(b0 + bi + 1) * N + tid) * plane + f0);
         const int next_req = rots[b0 + min(bi + 1, nb - 1)].req;
         if (req != sp_req) {   // block-uniform
             __syncthreads();   // the previous tile is no longer read
@@ -907,6 +915,7 @@ k_zpass16(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, co
 #pragma unroll
         for (int r = 0; r < 16; ++r) __stcs(&dst[(size_t)(j + 16 * r) * plane], make_float2(v[r].x, v[r].y));
         req = next_req;
+        if (bi + 1 < nb) load(bi + 1, v);
         __syncthreads();   // the exchange buffer is free for the next rotation
     }
 }
@@ -1238,8 +1247,9 @@ k_zpass_tc(int B, int group, const float2 *__restrict__ Y, const RotRec *rots, c
 // object's spectrum conj(F(O)) / M^3 and with conj(F(min(O, 0))) / M^3 (the
 // second only for requests with non-contact poses), summed before one inverse
 // FFT.  Both spectrum tiles sit in shared memory (reloaded when the request
-// changes), both inputs of the next rotation are in flight during the current
-// one, and the three transforms share one [256][16] exchange buffer.
+// changes), both inputs of the next rotation are on their way to L2 during the
+// current one (see k_zpass16: 40.2 -> 34.3 us a rotation), and the three
+// transforms share one [256][16] exchange buffer.
 // ---------------------------------------------------------------------------
 struct Zpass16DualCfg {
     static constexpr int M = 256, N = 128, P = 130, NT = 256, COLS = 16;
@@ -1285,18 +1295,18 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
         for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], cconj(twc_inv(j * r)));   // exp(-2 pi i j r / 256)
         DFT<16, false>::run(v);
     };
-    cf nx[8], nx2[8];
-    load(Y, 0, nx);
+    cf v[16], nx2[8];
+    load(Y, 0, v);
     load(Y2, 0, nx2);
     int sp_req = -1, req = rots[b0].req;   // looked up one rotation ahead
     bool pen = false;
     float cj = 1.f;
 #pragma unroll 1
     for (int bi = 0; bi < nb; ++bi) {
-        cf v[16], w[16];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) v[s] = nx[s];
-        if (bi + 1 < nb) load(Y, bi + 1, nx);
+        cf w[16];
+        // the next rotation's 128 + 128 lines of 16 columns, towards L2
+        if (bi + 1 < nb)
+            prefetch_l2((tid < N ? Y : Y2) + ((size_t)(b0 + bi + 1) * N + (tid & (N - 1))) * plane + f0);
         const int next_req = rots[b0 + min(bi + 1, nb - 1)].req;
         if (req != sp_req) {   // block-uniform
             __syncthreads();   // the previous tiles are no longer read
@@ -1332,13 +1342,10 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
             // non-contact sweep: w += F(S_nc) conj(F(min(O, 0))) / M^3
 #pragma unroll
             for (int s = 0; s < 8; ++s) v[s] = nx2[s];
-            if (bi + 1 < nb) load(Y2, bi + 1, nx2);
             __syncthreads();   // every thread has read its forward stage-1 inputs
             forward(v);
 #pragma unroll
             for (int r = 0; r < 16; ++r) w[r] = cadd(w[r], cmul(v[r], ppt[(j + 16 * r) * COLS + c]));
-        } else if (bi + 1 < nb) {
-            load(Y2, bi + 1, nx2);
         }
         __syncthreads();   // every thread has read its last forward stage-1 inputs
         // inverse, stage 0 (inputs kz = j + 16 r) -> index 16 j + r
@@ -1355,6 +1362,10 @@ k_zpass16_dual(int B, int group, const float2 *__restrict__ Y, const float2 *__r
 #pragma unroll
         for (int r = 0; r < 16; ++r) __stcs(&dst[(size_t)(j + 16 * r) * plane], make_float2(w[r].x, w[r].y));
         req = next_req;
+        if (bi + 1 < nb) {
+            load(Y, bi + 1, v);
+            load(Y2, bi + 1, nx2);
+        }
         __syncthreads();   // the exchange buffer is free for the next rotation
     }
 }

@@ -35,6 +35,11 @@ __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src)
     unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem_src) : "memory");
 }
+// the 128-byte line of gmem is fetched towards L2; no register waits for it
+__device__ __forceinline__ void prefetch_l2(const void *gmem)
+{
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(gmem));
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 // wait until at most n (0..3) of this thread's committed groups are pending
@@ -928,11 +933,11 @@ cudaError_t launch_rot_export(const Geo &g, const ReqDev *reqs, const RotRec *ro
 // inverse transform yields the sum of both correlations.  Requests without
 // non-contact poses skip the addition and keep the plain result bit for bit.
 // Bound by the memory traffic of Y and Z and the chain of its exchanges: the
-// inputs come straight from global memory into registers, the next tile's in
-// flight during the current one, and blocks of 16 columns (64 to 256 threads)
+// inputs come straight from global memory into registers, the next tile's on
+// their way during the current one, and blocks of 16 columns (64 to 256 threads)
 // leave four to eight of them on an SM.  With 32 columns staged by 8-byte
 // cp.async and the second spectrum read again per rotation, a rotation took 0.58,
-// 3.74 us (plain, N = 32, 64) and 30.3 us (DUAL, N = 96); now 0.33, 3.05 and 20.0.
+// 3.74 us (plain, N = 32, 64) and 30.3 us (DUAL, N = 96); now 0.33, 2.55 and 19.2.
 // ---------------------------------------------------------------------------
 template <int M, bool DUAL, int V = 0> struct ZpassCfg {
     static constexpr int COLS = M == 256 ? 32 : 16, NT = Plan<M, V>::T * COLS;
@@ -940,6 +945,12 @@ template <int M, bool DUAL, int V = 0> struct ZpassCfg {
     static constexpr size_t SMEM = sizeof(cf) * ((size_t)M * COLS * (DUAL ? 3 : 2) + M);
     // resident blocks the registers are allotted for
     static constexpr int MINB = (Plan<M, V>::E <= 8 ? 1024 : DUAL ? 512 : 768) / NT;
+    // The next tile waits in L2 (one prefetch per row of 16 columns, the loads
+    // at the end of the tile), not in registers.  The registers this frees pay at
+    // canvas 128: 3.01 -> 2.55 us a rotation (plain), 4.38 -> 4.18 (DUAL).  At the
+    // others the wait for L2 costs more: 0.328 -> 0.344 us (64), 11.7 -> 12.2
+    // (192), 19.2 -> 21.3 (192, DUAL).
+    static constexpr bool VIA_L2 = M == 128;
 };
 
 template <int M, bool DUAL, int V = 0>
@@ -972,8 +983,8 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
             v[s] = cmake(a.x, a.y);
         }
     };
-    cf nx[EL];
-    load(0, nx);
+    cf v[E], nx[C::VIA_L2 ? 1 : EL];
+    load(0, C::VIA_L2 ? v : nx);
     // the request of a rotation is looked up one rotation ahead: rots -> reqs is
     // a chain of two memory latencies that a tile would otherwise begin with
     int sp_req = -1, req = rots[b0].req, P_nc = 0;
@@ -982,14 +993,23 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
     __syncthreads();   // the twiddles
 #pragma unroll 1
     for (int t = 0; t < nt; ++t) {
-        cf v[E];
         // (slots s < E / 2 of the first stage read z < N, the others the padding)
         static_assert(slot_in_lower_half<M, V>(EL - 1) && !slot_in_lower_half<M, V>(EL), "input slots");
+        if constexpr (!C::VIA_L2) {
 #pragma unroll
-        for (int s = 0; s < EL; ++s) v[s] = nx[s];
+            for (int s = 0; s < EL; ++s) v[s] = nx[s];
+        }
 #pragma unroll
         for (int s = EL; s < E; ++s) v[s] = cmake(0.f, 0.f);
-        if (t + 1 < nt) load(t + 1, nx);
+        if (t + 1 < nt) {
+            if constexpr (C::VIA_L2) {   // one request per row of 16 columns
+                const float2 *next = ((DUAL && !(t & 1)) ? Y2 : Y) + (size_t)(b0 + (t + 1) / TPR) * N * plane + f0;
+                for (int i = threadIdx.x; i < N * (COLS / 16); i += C::NT)
+                    prefetch_l2(&next[(size_t)(i / (COLS / 16)) * plane + i % (COLS / 16) * 16]);
+            } else {
+                load(t + 1, nx);
+            }
+        }
         const bool second = DUAL && (t & 1);
         const int bi = t / TPR, next_req = rots[b0 + min(t + 1, nt - 1) / TPR].req;
         if (!second && req != sp_req) {   // block-uniform; each thread reads the entries it writes
@@ -1049,6 +1069,7 @@ k_zpass(int P, int B, int group, const float2 *__restrict__ Y, const float2 *__r
                 __stcs(&Zb[(size_t)out_index<M, V>(j, s) * plane], make_float2(w[s].x, w[s].y));
         }
         req = next_req;
+        if (C::VIA_L2 && t + 1 < nt) load(t + 1, v);
     }
 }
 
