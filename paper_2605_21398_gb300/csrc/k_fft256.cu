@@ -479,7 +479,7 @@ k_plane_ps(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUt
     // the key of the plane's rotation.  Its address is a chain of two memory
     // latencies (rots -> reqs): looked up while the plane's columns arrive and
     // kept until the plane's key has left, so that no wait of phase 2 or of the
-    // flush begins with it.
+    // flush begins with it (35.7 -> 35.1 us a rotation).
     unsigned long long *rot_key = nullptr;
     bool key_waits = false;   // (thread 0) the previous plane's key is in s_key
     // the previous plane's key (every warp has added to it before the barrier
