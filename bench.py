@@ -266,13 +266,14 @@ def serving_experiment(ctx, synth):
 
 
 # Per-rotation counters of the search kernels as they are now, from one ncu capture each of an
-# 8-rotation launch of `bench.py --ncu-case` (dram__bytes_read.sum + dram__bytes_write.sum, and
-# smsp__inst_executed.sum for the voxeliser); a launch of B rotations is scaled from them by B/8
+# 8-rotation launch of `bench.py --ncu-case` (dram__bytes_read.sum + dram__bytes_write.sum); a launch of B rotations is scaled from them by B/8
 # (the z pass adds one spectrum read per launch).  A kernel changed since its capture has no entry.
-# That z pass launch has three blocks per block column, each reading the spectrum once.
+# That z pass launch has three blocks per block column, each reading the spectrum once.  The
+# voxeliser's smsp__inst_executed.sum is over a search of 256 SF rotations of the same workload (20 to 39 M
+# a rotation).
 NCU_DRAM_BYTES_PER_ROT = {"plane": (545357312 + 3463168) / 8, "fwd2d": (18613248 + 229198848) / 8,
                           "zpass": (476177920 - 3 * 68157440 + 485797888) / 8, "voxelise": (908288 + 0) / 8}
-NCU_WARP_INST_PER_ROT = {"voxelise": 240127528 / 8}
+NCU_WARP_INST_PER_ROT = {"voxelise": 6580964989 / 256}
 # SMs x warp schedulers: one warp instruction issued per scheduler per clock
 ISSUE_SLOTS = 152 * 4
 
@@ -595,7 +596,7 @@ def main():
         return {"bound": "alu", "kernel": k, "achieved": round(achieved, 1), "peak": round(pk, 1),
                 "unit": "G warp-instructions/s", "frac": round(achieved / pk, 4),
                 "traffic": int(NCU_DRAM_BYTES_PER_ROT[k] * rot_total / max(1, launches)),
-                "work_source": "smsp__inst_executed.sum of an 8-rotation ncu capture (%.1f M per rotation)"
+                "work_source": "smsp__inst_executed.sum over 256 rotations (%.1f M per rotation)"
                                % (NCU_WARP_INST_PER_ROT[k] / 1e6),
                 "peak_source": "152 SMs x 4 schedulers x %.0f MHz (maximum SM clock)" % sm_max_mhz()}
 
