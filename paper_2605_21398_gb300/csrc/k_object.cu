@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "dock_internal.h"
+#include "tri_f32.h"
 
 namespace dock {
 
@@ -208,89 +209,27 @@ k_object_rows(const double *V, const int32_t *T, ObjBins bins, int N, double h, 
     if ((kx & 31) == 0) inside[(size_t)blockIdx.x * (N / 32) + kx / 32] = w;
 }
 
-// A triangle in FP32 relative to the lattice origin: v0, the edges to v1 and
-// v2, its longest edge, and how far (mm) an FP32 distance to it may be off.
-struct TriF {
-    float v0[3], e0[3], e1[3], reach, tol;
-    int32_t touch;
-};
-static_assert(sizeof(TriF) == 48, "triangle record");
-
 size_t tri_f32_bytes() { return sizeof(TriF); }
 
-// S: the lattice's extent; a coordinate relative to its origin is rounded to
-// 2^-24 S (point and vertex).  A normal of a triangle of altitude a turns by
-// that over a, which moves a plane distance measured from up to 2 cut + edge
-// away; degenerate triangles get an infinite tolerance.
 __global__ void k_tri_f32(int n, const double *V, const int32_t *T, const uint8_t *touch, double o0, double o1,
                           double o2, float S, float cut, TriF *out)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     const double o[3] = {o0, o1, o2};
-    float v[3][3];
+    double v[3][3];
     for (int m = 0; m < 3; ++m)
-        for (int a = 0; a < 3; ++a) v[m][a] = (float)(V[3 * (size_t)T[3 * t + m] + a] - o[a]);
-    TriF r;
-    float l0 = 0.f, l1 = 0.f, l2 = 0.f;
-    for (int a = 0; a < 3; ++a) {
-        r.v0[a] = v[0][a];
-        r.e0[a] = v[1][a] - v[0][a];
-        r.e1[a] = v[2][a] - v[0][a];
-        const float d = v[2][a] - v[1][a];
-        l0 += r.e0[a] * r.e0[a];
-        l1 += r.e1[a] * r.e1[a];
-        l2 += d * d;
-    }
-    const float n0 = r.e0[1] * r.e1[2] - r.e0[2] * r.e1[1], n1 = r.e0[2] * r.e1[0] - r.e0[0] * r.e1[2];
-    const float n2 = r.e0[0] * r.e1[1] - r.e0[1] * r.e1[0];
-    const float edge = sqrtf(fmaxf(l0, fmaxf(l1, l2))), area = sqrtf(n0 * n0 + n1 * n1 + n2 * n2);
-    const float delta = 5e-7f * S, far = 2.f * cut + edge;
-    // the altitude itself is uncertain by a few delta
-    const float alt = edge > 0.f ? area / edge - 8.f * delta : 0.f;
-    r.reach = edge + 4.f * delta;
-    r.tol = alt > 0.f ? 4.f * delta * (1.f + far / alt) : INFINITY;
-    r.touch = (touch == nullptr || touch[t]) ? 1 : 0;
-    out[t] = r;
-}
-
-// FP32 distance from p (relative to the lattice origin) to a triangle: the
-// smallest of the three edges' and, when the projection falls inside, the
-// plane's.  INFINITY when farther than `skip` (a bound on what matters).
-__device__ __forceinline__ float tri_dist_f32(const TriF &t, float px, float py, float pz, float skip)
-{
-    const float w0 = px - t.v0[0], w1 = py - t.v0[1], w2 = pz - t.v0[2];
-    const float ww = fmaf(w0, w0, fmaf(w1, w1, w2 * w2)), lim = skip + t.reach;
-    if (ww > lim * lim) return INFINITY;
-    const float *a = t.e0, *b = t.e1;
-    const float aa = fmaf(a[0], a[0], fmaf(a[1], a[1], a[2] * a[2])), bb = fmaf(b[0], b[0], fmaf(b[1], b[1], b[2] * b[2]));
-    const float ab = fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2]));
-    const float wa = fmaf(w0, a[0], fmaf(w1, a[1], w2 * a[2])), wb = fmaf(w0, b[0], fmaf(w1, b[1], w2 * b[2]));
-    // nearest point of each edge: w - t e
-    auto off = [&](float s, float u) -> float {   // |w - s a - u b|^2
-        const float q0 = w0 - fmaf(s, a[0], u * b[0]), q1 = w1 - fmaf(s, a[1], u * b[1]), q2 = w2 - fmaf(s, a[2], u * b[2]);
-        return fmaf(q0, q0, fmaf(q1, q1, q2 * q2));
-    };
-    const float sa = aa > 0.f ? fminf(1.f, fmaxf(0.f, wa / aa)) : 0.f;
-    const float sb = bb > 0.f ? fminf(1.f, fmaxf(0.f, wb / bb)) : 0.f;
-    // edge v1 v2: points (1 - s) a + s b
-    const float cc = aa - 2.f * ab + bb, wc = (wb - wa) - (ab - aa);
-    const float sc = cc > 0.f ? fminf(1.f, fmaxf(0.f, wc / cc)) : 0.f;
-    float d2 = fminf(off(sa, 0.f), fminf(off(0.f, sb), off(1.f - sc, sc)));
-    const float den = fmaf(aa, bb, -ab * ab), u = fmaf(bb, wa, -ab * wb), v = fmaf(aa, wb, -ab * wa);
-    if (den > 0.f && u >= 0.f && v >= 0.f && u + v <= den) {
-        const float n0 = a[1] * b[2] - a[2] * b[1], n1 = a[2] * b[0] - a[0] * b[2], n2 = a[0] * b[1] - a[1] * b[0];
-        const float nn = fmaf(n0, n0, fmaf(n1, n1, n2 * n2)), wn = fmaf(w0, n0, fmaf(w1, n1, w2 * n2));
-        if (nn > 0.f) d2 = fminf(d2, wn * wn / nn);
-    }
-    return sqrtf(d2);
+        for (int a = 0; a < 3; ++a) v[m][a] = V[3 * (size_t)T[3 * t + m] + a] - o[a];
+    out[t] = tri_f32(v, S, cut, touch == nullptr || touch[t]);
 }
 
 // One block per bin cell: band values of the cell's voxels.  FP64 operations
 // run at a 64th of the FP32 rate, so the triangles of the cell (about 500 near
 // a surface of 65 k triangles) are measured in FP32 first, and the exact FP64
-// distance (whose minimum is the result) is formed only for those that the FP32
-// distance and its error bound leave in question, a few per voxel.  Two
+// distance (whose minimum is the result) is formed only for those whose FP32
+// lower bound does not lie above the smallest FP32 upper bound, a few per voxel
+// (tri_f32.h: bounds for triangles of any shape; the thinnest always get their
+// FP64 distance).  Two
 // threads per voxel share the triangles of a tile; the voxel-triangle pairs in
 // question are dealt to the block.  44.2 -> 3.1 ms (rows and cells) at N = 128 and 65 k triangles
 // (with one thread per voxel and FP64 throughout, lanes of a warp walking
@@ -299,8 +238,8 @@ __device__ __forceinline__ float tri_dist_f32(const TriF &t, float px, float py,
 // each, the axes one after another).
 __global__ void __launch_bounds__(128)
 k_object_cells(const double *V, const int32_t *T, const TriF *tri, ObjBins bins, const int32_t *axis, int N, double h,
-               double o0, double o1, double o2, double tau_out, double tau_in, double deep, const uint32_t *inside,
-               float *O)
+               double o0, double o1, double o2, double tau_out, double tau_in, double deep, float edge_tol,
+               const uint32_t *inside, float *O)
 {
     constexpr int NT = 128, NV = 64, TILE = 64, PAIRS = 4096, ROOM = 8 * NT;
     __shared__ TriF tile[TILE];
@@ -338,8 +277,14 @@ k_object_cells(const double *V, const int32_t *T, const TriF *tri, ObjBins bins,
     for (int base = 0; base < nv; base += NV) {
         const int s = tid >> 1, half = tid & 1, v = base + s;
         const bool on = v < nv;
-        const float px = (float)(h * (double)(x0 + v % lx)), py = (float)(h * (double)(y0 + (v / lx) % ly));
-        const float pz = (float)(h * (double)(z0 + v / (lx * ly)));
+        // relative to the origin, as the FP64 point rounds (for the warps that have a voxel: FP64
+        // operations are what a cell of one voxel and no triangle costs)
+        float px = 0.f, py = 0.f, pz = 0.f;
+        if (on) {
+            px = (float)((h * (double)(x0 + v % lx) + o0) - o0);
+            py = (float)((h * (double)(y0 + (v / lx) % ly) + o1) - o1);
+            pz = (float)((h * (double)(z0 + v / (lx * ly)) + o2) - o2);
+        }
         if (tid < NV) best[tid] = bestt[tid] = 0x7FF0000000000000ull;   // +infinity
         if (tid == 0) n_pairs = 0;
         // pass 0: upper bounds of the two minima; pass 1: the pairs in question
@@ -352,27 +297,31 @@ k_object_cells(const double *V, const int32_t *T, const TriF *tri, ObjBins bins,
                 __syncthreads();
                 for (int k = tid; k < nt; k += NT) tidx[k] = bins.cell3_items[i0 + j0 + k];
                 __syncthreads();
-                for (int k = tid; k < nt * 12; k += NT)
-                    reinterpret_cast<uint32_t *>(tile)[k] = reinterpret_cast<const uint32_t *>(tri + tidx[k / 12])[k % 12];
+                constexpr int W = sizeof(TriF) / 4;
+                for (int k = tid; k < nt * W; k += NT)
+                    reinterpret_cast<uint32_t *>(tile)[k] = reinterpret_cast<const uint32_t *>(tri + tidx[k / W])[k % W];
                 __syncthreads();
                 for (int k0 = 0; k0 < nt; k0 += 16) {
                     // eight triangles of the tile per thread, then room is looked for again
                     if (on)
                         for (int k = k0 + half; k < min(nt, k0 + 16); k += 2) {
                             const TriF &t = tile[k];
-                            // (a triangle without a usable FP32 distance is always in question)
+                            // (a triangle without a usable FP32 bound is always in question)
                             const bool sure = t.tol < INFINITY;
                             const float b = fminf(skip, fmaxf(ub, ubt));
-                            const float d = sure ? tri_dist_f32(t, px, py, pz, b + t.tol) : 0.f;
                             if (pass == 0) {
                                 if (sure) {
-                                    ub = fminf(ub, d + t.tol);
-                                    if (t.touch) ubt = fminf(ubt, d + t.tol);
+                                    const float d = tri_bound_f32<true>(t, px, py, pz, b, edge_tol) + edge_tol;
+                                    ub = fminf(ub, d);
+                                    if (t.touch) ubt = fminf(ubt, d);
                                 }
-                            } else if (!sure || d - t.tol <= fminf(skip, ub) || (t.touch && d - t.tol <= fminf(skip, ubt))) {
-                                const int k2 = atomicAdd(&n_pairs, 1);
-                                pair_i[k2] = j0 + k;
-                                pair_s[k2] = (unsigned char)s;
+                            } else {
+                                const float d = sure ? tri_bound_f32<false>(t, px, py, pz, b, edge_tol) : 0.f;
+                                if (!sure || d <= fminf(skip, ub) || (t.touch && d <= fminf(skip, ubt))) {
+                                    const int k2 = atomicAdd(&n_pairs, 1);
+                                    pair_i[k2] = j0 + k;
+                                    pair_s[k2] = (unsigned char)s;
+                                }
                             }
                         }
                     if (pass == 1) {
@@ -417,11 +366,11 @@ cudaError_t launch_object_grid(const double *V, const int32_t *T, int64_t nt, co
 {
     TriF *tf = static_cast<TriF *>(tri);
     const double cut = tau_out > tau_in ? tau_out : tau_in;
-    k_tri_f32<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>((int)nt, V, T, touch, o[0], o[1], o[2], (float)(N * h),
-                                                            (float)cut, tf);
+    const float S = (float)(N * h);
+    k_tri_f32<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>((int)nt, V, T, touch, o[0], o[1], o[2], S, (float)cut, tf);
     k_object_rows<<<N * N, 128, 0, st>>>(V, T, bins, N, h, o[0], o[1], o[2], inside, err);
     k_object_cells<<<bins.d3[0] * bins.d3[1] * bins.d3[2], 128, 0, st>>>(V, T, tf, bins, axis, N, h, o[0], o[1], o[2],
-                                                                        tau_out, tau_in, deep, inside, O);
+                                                                        tau_out, tau_in, deep, tri_edge_tol(S), inside, O);
     return cudaGetLastError();
 }
 
