@@ -200,7 +200,9 @@ DOCK_API const char *dock_version(void);
  *   o_o      = h round(c / h) - (N/2) h, c = the mesh AABB centre.
  * The SDF is the exact point-triangle distance with the sign from the parity
  * of +x ray crossings.  Returns DOCK_E_INVALID when the mesh AABB widened by
- * tau_out1 does not fit the lattice.  Also builds the BVH used by the
+ * tau_out1 does not fit the lattice, and DOCK_E_TOO_LARGE when its triangles'
+ * boxes (widened by the larger band) meet more than 2^31 - 1 cells, of side
+ * max(h, tau_out1, tau_in1), in all.  Also builds the BVH used by the
  * refinement (Sec. V-B) and sets the anchor a = AABB centre (Sec. V-A).
  */
 DOCK_API dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int64_t V, const int32_t *tris, int64_t T,

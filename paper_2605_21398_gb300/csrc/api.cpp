@@ -825,6 +825,7 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     double *dV = nullptr;
     int32_t *dT = nullptr, *ds3 = nullptr, *di3 = nullptr, *ds2 = nullptr, *di2 = nullptr, *at3 = nullptr, *at2 = nullptr;
     int32_t *dorder = nullptr, *dwhich = nullptr, *daxis = nullptr;
+    unsigned long long *dtotal = nullptr;
     BvhNode *dnodes = nullptr;
     void *dtri = nullptr;
     uint32_t *dinside = nullptr;
@@ -842,18 +843,23 @@ extern "C" dock_status dock_object_grid(dock_ctx *ctx, const double *verts, int6
     ds2 = ds3 + n3 + 1;
     at3 = ds2 + n2 + 1;
     at2 = at3 + n3 + 1;
+    if ((s = temp(&dtotal, sizeof(unsigned long long) * 2)) != DOCK_OK) return bail(s);
     CKB(cudaMemcpyAsync(dV, verts, sizeof(double) * 3 * V, cudaMemcpyHostToDevice, st));
     CKB(cudaMemcpyAsync(dT, tris, sizeof(int32_t) * 3 * T, cudaMemcpyHostToDevice, st));
     CKB(cudaMemsetAsync(ds3, 0, sizeof(int32_t) * (n3 + 1 + n2 + 1), st));
+    unsigned long long total[2] = {0, 0};
+    CKB(cudaMemsetAsync(dtotal, 0, sizeof(total), st));
+    CKB(launch_bins_total(dV, dT, T, ob->o, cs, d3, cut, dtotal, st));
+    CKB(cudaMemcpyAsync(total, dtotal, sizeof(total), cudaMemcpyDeviceToHost, st));
+    CKB(cudaStreamSynchronize(st));
+    if (total[0] > INT32_MAX || total[1] > INT32_MAX)
+        return bail(fail(ctx, DOCK_E_TOO_LARGE, "%lld triangles meet %llu bin cells: more than 2^31 - 1", (long long)T,
+                         std::max(total[0], total[1])));
     CKB(launch_bins_count(dV, dT, T, ob->o, cs, d3, false, cut, ds3, st));
     CKB(launch_bins_count(dV, dT, T, ob->o, cs, d3, true, 0.0, ds2, st));
     CKB(cudaMemcpyAsync(at3, ds3, sizeof(int32_t) * (n3 + 1 + n2 + 1), cudaMemcpyDeviceToDevice, st));
-    int32_t total3 = 0, total2 = 0;
-    CKB(cudaMemcpyAsync(&total3, ds3 + n3, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    CKB(cudaMemcpyAsync(&total2, ds2 + n2, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    CKB(cudaStreamSynchronize(st));
-    if ((s = temp(&di3, sizeof(int32_t) * std::max(1, total3))) != DOCK_OK) return bail(s);
-    if ((s = temp(&di2, sizeof(int32_t) * std::max(1, total2))) != DOCK_OK) return bail(s);
+    if ((s = temp(&di3, sizeof(int32_t) * std::max(1ull, total[0]))) != DOCK_OK) return bail(s);
+    if ((s = temp(&di2, sizeof(int32_t) * std::max(1ull, total[1]))) != DOCK_OK) return bail(s);
     if ((s = temp(&dtri, tri_f32_bytes() * T)) != DOCK_OK) return bail(s);
     if ((s = temp(&dinside, sizeof(uint32_t) * (size_t)N * N * (N / 32))) != DOCK_OK) return bail(s);
     if ((s = temp(&daxis, sizeof(int32_t) * axis.size())) != DOCK_OK) return bail(s);

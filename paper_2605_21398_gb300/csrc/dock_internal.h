@@ -148,8 +148,13 @@ cudaError_t launch_rot_export(const Geo &g, const ReqDev *reqs, const RotRec *ro
 
 // Object grid kernels (k_object.cu)
 // Bins of triangles over cells of side cs, CSR: per triangle the cells its box
-// (widened by pad) meets; cells over (x, y, z), or over (y, z) when flat.  count: n_cells + 1 zeros in, exclusive prefix sums out (the total at
-// the end); fill writes the items, `at` being a copy of the prefix sums.
+// (widened by pad) meets; cells over (x, y, z), or over (y, z) when flat.  total: adds the
+// number of entries of both to total[0] (pad) and total[1] (flat, no pad), in 64 bits; the
+// others count in 32 and are called when both fit.  count: n_cells + 1 zeros in, exclusive
+// prefix sums out (the total at the end); fill writes the items, `at` being a copy of the
+// prefix sums.
+cudaError_t launch_bins_total(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                              double pad, unsigned long long *total, cudaStream_t st);
 cudaError_t launch_bins_count(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
                               bool flat, double pad, int32_t *start, cudaStream_t st);
 cudaError_t launch_bins_fill(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,

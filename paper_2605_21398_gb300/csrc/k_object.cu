@@ -91,6 +91,31 @@ __device__ __forceinline__ bool tri_cells(const double *V, const int32_t *T, int
     return true;
 }
 
+// total[0] += the entries of the 3-D bins, total[1] += those of the (y, z) bins
+__global__ void k_bins_total(const double *V, const int32_t *T, int64_t nt, double3 o, double cs, int3 d, double pad,
+                             unsigned long long *total)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long n[2] = {0ull, 0ull};
+    int lo[3], hi[3];
+    if (t < nt && tri_cells(V, T, t, o, cs, d, false, pad, lo, hi))
+        n[0] = (unsigned long long)(hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
+    if (t < nt && tri_cells(V, T, t, o, cs, d, true, 0.0, lo, hi))
+        n[1] = (unsigned long long)(hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
+    for (int k = 0; k < 2; ++k) {
+        for (int s = 16; s > 0; s >>= 1) n[k] += __shfl_down_sync(0xFFFFFFFFu, n[k], s);
+        if ((threadIdx.x & 31) == 0 && n[k]) atomicAdd(&total[k], n[k]);
+    }
+}
+
+cudaError_t launch_bins_total(const double *V, const int32_t *T, int64_t nt, const double *o, double cs, const int *d,
+                              double pad, unsigned long long *total, cudaStream_t st)
+{
+    k_bins_total<<<(unsigned)((nt + 127) / 128), 128, 0, st>>>(V, T, nt, make_double3(o[0], o[1], o[2]), cs,
+                                                               make_int3(d[0], d[1], d[2]), pad, total);
+    return cudaGetLastError();
+}
+
 // at[cell] += 1 per triangle and cell; with items given, the old value is the
 // triangle's place (the order within a cell does not matter: minima and
 // parities are taken over it)
