@@ -50,3 +50,16 @@ def test_boxes_that_span_the_lattice(ctx):
     G, _ = ob.export_grid()
     Go, _, _, fits = O.object_grid(V, T, 0.6, 128)
     assert fits and np.array_equal(G, Go.astype(np.float32))
+
+
+@pytest.mark.parametrize("N, h", [(32, 0.6), (64, 0.3), (96, 0.5), (128, 0.15)])
+@pytest.mark.parametrize("n", [2, 15, 16, 70])
+def test_boxes_shared_by_a_warp_and_its_parts(ctx, N, h, n):
+    # 4 to 140 triangles: a part of a warp, whole warps and a part, more than a block
+    half = 0.5 * (N - 1) * h - 1.6
+    V, T = _rod(max(n, 3), half, 0.7)
+    V, T = V @ synth.quat_to_mat(synth.random_quat(np.random.default_rng(n))).T * 0.55, T[:2 * n]
+    ob = ctx.object_grid(V, T, h, N)
+    G, _ = ob.export_grid()
+    Go, _, _, fits = O.object_grid(V, T, h, N)
+    assert fits and np.array_equal(G, Go.astype(np.float32))
