@@ -1290,10 +1290,13 @@ k_refine_dist(const RefineDev *Dt, const int32_t *grp, const CandF *cands, doubl
         PoseTerms o;
         if (mine) {
             const unsigned long long key = S.sbest[tid], all = S.best[tid];
-            // the strict candidates hold the smallest d, and none of the
-            // bounds met can have hidden the one that does
-            const float dall = unord_f((uint32_t)(all >> 32));
-            bool hidden = all != ~0ull && dall <= eps && (uint32_t)(key >> 32) != (uint32_t)(all >> 32);
+            // the strict candidates hold the smallest d, none of the bounds met
+            // can have hidden the one that does, and the smallest value found
+            // lies at the bound that ruled the others out: on triangles of many
+            // millimetres a search may end 1e-4 above a point that gave the bound
+            const float dall = all != ~0ull ? unord_f((uint32_t)(all >> 32)) : INFINITY, lim = unord_f(S.lim[tid]);
+            bool hidden = (dall <= eps && (uint32_t)(key >> 32) != (uint32_t)(all >> 32)) ||
+                          (lim <= eps && dall > lim + 0.5f * S.fr[tid][12]);
             const bool hit = key != ~0ull;
             float lv[3][3], xl[3] = {0.f, 0.f, 0.f};
             if (hit) {
@@ -1302,7 +1305,7 @@ k_refine_dist(const RefineDev *Dt, const int32_t *grp, const CandF *cands, doubl
                 const float u = S.wu[tid], v = S.wv[tid], w0 = 1.f - u - v;
                 for (int a = 0; a < 3; ++a) xl[a] = fmaf(w0, lv[0][a], fmaf(u, lv[1][a], v * lv[2][a]));
                 newhint = pack_hint(S.wslot[tid], u, v);
-                if (dall <= eps && S.wslot[tid] != S.hslot[tid] && lin_lower_bound(lv, D.r, D.L) > unord_f(S.lim[tid]))
+                if (dall <= eps && S.wslot[tid] != S.hslot[tid] && lin_lower_bound(lv, D.r, D.L) > lim)
                     hidden = true;
             }
             if (hidden) S0->redo[row / 32] = 1;
@@ -1343,8 +1346,8 @@ k_refine_dist(const RefineDev *Dt, const int32_t *grp, const CandF *cands, doubl
 // around the vertex can exceed the vertex's own value by its rounding (one pose
 // in 1e5 at a contact of a flat face).  What is then reported, the next best
 // triangle or none, depends on the order of the walk.  k_refine_dist sees these
-// cases (the smallest d belongs to a triangle its own bound rules out) and
-// lists their 32 poses; here one warp walks for 32 poses together, entering a
+// cases (the smallest d belongs to a triangle its own bound rules out, or lies
+// above the bound that ruled out others) and lists their 32 poses; here one warp walks for 32 poses together, entering a
 // node when any lane needs it, the nearer child (by the smallest bound over the
 // lanes) first, and settles a lane's triangles in the order of their bounds.
 // The list is short (about 5 of 10000 warps on a first evaluation of 64 x 5000
