@@ -29,6 +29,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "dock_internal.h"
 
 namespace cg = cooperative_groups;
@@ -1308,7 +1310,9 @@ k_refine_dist(const RefineDev *Dt, const int32_t *grp, const CandF *cands, doubl
                 if (dall <= eps && S.wslot[tid] != S.hslot[tid] && lin_lower_bound(lv, D.r, D.L) > lim)
                     hidden = true;
             }
-            if (hidden) S0->redo[row / 32] = 1;
+            // (beyond the cutoff the score is zero; where the distance itself is asked for, it is that of
+            // the triangles its shared walk meets)
+            if (hidden || (dist_out && !(dall <= eps))) S0->redo[row / 32] = 1;
             pose_terms<GRAD>(D, cf, D.poses[i], hit, hit ? unord_f((uint32_t)(key >> 32)) : INFINITY, xl, lv,
                              (size_t)c * D.P + i, dist_out, wit_out, nrm_out, o);
         }
@@ -1347,7 +1351,10 @@ k_refine_dist(const RefineDev *Dt, const int32_t *grp, const CandF *cands, doubl
 // in 1e5 at a contact of a flat face).  What is then reported, the next best
 // triangle or none, depends on the order of the walk.  k_refine_dist sees these
 // cases (the smallest d belongs to a triangle its own bound rules out, or lies
-// above the bound that ruled out others) and lists their 32 poses; here one warp walks for 32 poses together, entering a
+// above the bound that ruled out others) and lists their 32 poses.  Beyond the cutoff, too, what is reported is the nearest
+// of the triangles that the walk met on behalf of any of the 32 poses and that
+// pass the pose's own Eq. (21) test: dock_distances, which returns it, lists
+// those groups as well.  Here one warp walks for 32 poses together, entering a
 // node when any lane needs it, the nearer child (by the smallest bound over the
 // lanes) first, and settles a lane's triangles in the order of their bounds.
 // The list is short (about 5 of 10000 warps on a first evaluation of 64 x 5000
@@ -2003,9 +2010,11 @@ static cudaError_t launch_dist_t(const RefineDev *Dt, const int32_t *grp, int K,
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_refine_dist<Q, GRAD>, Dt, grp, cands, acc_part, nwarp, dist_out, wit_out,
                                        nrm_out, hints, active, redo);
     if (e != cudaSuccess) return e;
-    // two one-warp blocks per SM; an empty list costs the launch
-    k_refine_ordered<GRAD><<<2 * 152, 32, 0, st>>>(Dt, grp, cands, acc_part, nwarp, dist_out, wit_out, nrm_out, hints,
-                                                   redo);
+    // two one-warp blocks per SM (an empty list costs the launch); where distances are
+    // asked for, every group with a pose beyond the cutoff is on the list
+    const int blocks = dist_out ? (int)std::min<int64_t>((int64_t)K * nwarp, 32 * 152) : 2 * 152;
+    k_refine_ordered<GRAD><<<blocks, 32, 0, st>>>(Dt, grp, cands, acc_part, nwarp, dist_out, wit_out, nrm_out, hints,
+                                                  redo);
     return cudaGetLastError();
 }
 
