@@ -267,8 +267,8 @@ def serving_experiment(ctx, synth):
 
 # Per-rotation counters of the search kernels as they are now, from one ncu capture each of an
 # 8-rotation launch of `bench.py --ncu-case` (dram__bytes_read.sum + dram__bytes_write.sum); a launch of B rotations is scaled from them by B/8
-# (the z pass adds one spectrum read per launch).  A kernel changed since its capture has no entry.
-# That z pass launch has three blocks per block column, each reading the spectrum once.  The
+# (the z pass's spectrum reads apart: zpass_spectrum_reads).  A kernel changed since its capture has no entry.
+# That z pass launch has three blocks per block column, each reading its part of the spectrum once.  The
 # voxeliser's smsp__inst_executed.sum is over a search of 256 SF rotations of the same workload (20 to 39 M
 # a rotation).
 NCU_DRAM_BYTES_PER_ROT = {"plane": (545357312 + 3463168) / 8, "fwd2d": (18613248 + 229198848) / 8,
@@ -276,6 +276,16 @@ NCU_DRAM_BYTES_PER_ROT = {"plane": (545357312 + 3463168) / 8, "fwd2d": (18613248
 NCU_WARP_INST_PER_ROT = {"voxelise": 6580964989 / 256}
 # SMs x warp schedulers: one warp instruction issued per scheduler per clock
 ISSUE_SLOTS = 152 * 4
+
+
+def zpass_spectrum_reads(N, rots, tuning):
+    """How often a z pass launch of `rots` rotations reads the object's spectrum: every block along
+    the rotations reads its columns' part once.  The rotations of a block are the tuning's `group`,
+    or, when that is 0, the library's rule: about 5000 blocks in all, at most 16 rotations each."""
+    M, rots = 2 * N, max(1, int(round(rots)))
+    chunks = M * (N + 2) // (32 if M == 256 and tuning["zpass_cols"] == 32 else 16)
+    group = tuning["group"] or min(16, rots, chunks * rots // 5000)
+    return -(-rots // max(1, min(group, rots)))
 
 
 def max_over_ranks(ms, ws, device):
@@ -574,13 +584,13 @@ def main():
         M = 2 * w.N
         P = M // 2 + 2
         total_bytes = kernel_bytes(k, w.N) * rot_total
-        if k == "zpass":
-            total_bytes += M * M * P * 8 * launches   # spectrum read once per launch (block column)
-        achieved = total_bytes / (tot_ms / 1000.0) / 1e9
         rot_per_launch = rot_total / max(1, launches)
+        spectra = zpass_spectrum_reads(w.N, rot_per_launch, tuning) * M * M * P * 8 if k == "zpass" else 0
+        total_bytes += spectra * launches
+        achieved = total_bytes / (tot_ms / 1000.0) / 1e9
         traffic = None
         if k in NCU_DRAM_BYTES_PER_ROT:
-            traffic = NCU_DRAM_BYTES_PER_ROT[k] * rot_per_launch + (M * M * P * 8 if k == "zpass" else 0)
+            traffic = NCU_DRAM_BYTES_PER_ROT[k] * rot_per_launch + spectra
         return {"bound": "hbm", "kernel": k, "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": int(traffic) if traffic else None,
                 "traffic_source": "ncu capture of an 8-rotation launch, scaled to %.1f rotations per launch"

@@ -1348,9 +1348,9 @@ static dock_status run_pipeline_rots(dock_ctx *ctx, const Geo &g, const ReqDev *
     if (ro_any &&
         (s = ensure(ctx, (void **)&ctx->ogr, &ctx->ogr_n, (size_t)B * g.N * g.N * g.N, sizeof(float))) != DOCK_OK)
         return s;
-    // blocks of the z pass along the columns; about 5000 blocks in all keep the
-    // last wave small (at most 912 are resident), 16 rotations a block are enough
-    // to share a spectrum tile
+    // rotations per block of the z pass (a measured choice): about 5000 blocks in
+    // all, several waves, so that the last one is a small part of them; 16 rotations
+    // a block are enough to share a spectrum tile
     const int64_t chunks = (int64_t)g.M * g.P / (g.M == 256 && tc.zpass_cols == 32 ? 32 : 16);
     int k = 0;
     for (size_t b0 = r0; b0 < r1; b0 += B, ++k) {

@@ -18,12 +18,12 @@
 // the normal equations, trust-region scaling, box projection (Eq. (20)), and
 // the pose data of the next iteration (Eq. (14)-(17)).
 //
-// 21 evaluations and 20 steps on the GB300, one thread per pose before, now:
-// 8 x 200 poses 33.8 -> 4.0 ms, 64 x 5000 poses on 65 k triangles 262 -> 60 ms
-// (375 -> 60 on another object), 100 L-BFGS-B rounds of 32 x 2000 poses
-// 218 -> 34 ms.  Bound by the chain of a search (53 bisections of 20 steps, 156
-// cycles a step) while few poses run, by instruction issue (38 % of the slots)
-// and the last blocks' tail at 64 x 5000.
+// 21 evaluations and 20 steps on the GB300: 8 x 200 poses 4.0 ms, 64 x 5000 poses
+// on 65 k triangles 60 ms; 100 L-BFGS-B rounds of 32 x 2000 poses 36 ms.  Bound by
+// the chain of a search (53 bisections of 20 steps, 156 cycles a step) while few
+// poses run, by instruction issue (half of the slots), block barriers and the last
+// blocks' tail at 64 x 5000.  A thread per pose, its warp waiting for the longest of
+// 32 chains, takes 34, 262 to 375 and 218 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -2026,15 +2026,21 @@ cudaError_t launch_refine_eval(const RefineDev *Dt, const int32_t *grp, int K, i
     const size_t poses = (size_t)K * nwarp * 32;
     cudaError_t e0 = cudaMemsetAsync(redo, 0, sizeof(int32_t), st);
     if (e0 != cudaSuccess) return e0;
-#define DIST(Q)                                                                                                          return grad ? launch_dist_t<Q, true>(Dt, grp, K, nwarp, cands, acc_part, dist_out, wit_out, nrm_out, hints,                                               active, redo, st)                                                                              : launch_dist_t<Q, false>(Dt, grp, K, nwarp, cands, acc_part, dist_out, wit_out, nrm_out, hints,                                               active, redo, st);
+    const auto launch = [&](auto with_grad, auto without) {
+        return (grad ? with_grad : without)(Dt, grp, K, nwarp, cands, acc_part, dist_out, wit_out, nrm_out, hints,
+                                            active, redo, st);
+    };
     // Fewer poses per block while there are not enough blocks to fill the SMs
-    // (8: a cluster of four blocks shares a partial sum), 128 once there are:
-    // 21 evaluations of 1600 poses 3.5 / 4.3 / 7.7 ms at 8 / 32 / 128 poses per
-    // block, 100 of up to 64000 58 / 46 / 76 ms, 21 of 320000 169 / 98 / 82 ms.
-    if (poses <= 20000) { DIST(8) }
-    if (poses <= 200000) { DIST(32) }
-    DIST(128)
-#undef DIST
+    // (8: a cluster of four blocks shares a partial sum), 128 once there are.  The
+    // limits are those of L-BFGS-B, most of whose candidates are finished in most
+    // rounds: 100 rounds of up to 64000 queries 58 / 46 / 76 ms at 8 / 32 / 128 poses
+    // per block.  21 evaluations of Gauss-Newton, all of them active, on 65 k
+    // triangles: 2048 queries 4.0 / 4.9 / 9.1 ms, 5120 5.5 / 5.4 / 9.3, 19968 22.2 /
+    // 13.8 / 16.5, 40960 32 / 16.9 / 15.2, 198656 130 / 63 / 41, 327680 206 / 96 / 57:
+    // they would change over at 5000 and 30000.
+    if (poses <= 20000) return launch(launch_dist_t<8, true>, launch_dist_t<8, false>);
+    if (poses <= 200000) return launch(launch_dist_t<32, true>, launch_dist_t<32, false>);
+    return launch(launch_dist_t<128, true>, launch_dist_t<128, false>);
 }
 
 cudaError_t launch_refine_solve(int K, int nwarp, double *state, const double *acc_part, const double *prm, int mode,

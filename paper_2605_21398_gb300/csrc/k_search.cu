@@ -29,7 +29,7 @@ __device__ __forceinline__ double dm(double a, double b) { return __dmul_rn(a, b
 __device__ __forceinline__ double da(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double ds(double a, double b) { return __dsub_rn(a, b); }
 
-// asynchronous 8-byte global -> shared copies (completion: cp_async_wait_all)
+// asynchronous 8-byte global -> shared copies (completion: cp_async_commit, cp_async_wait_pending)
 __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src)
 {
     unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -41,7 +41,6 @@ __device__ __forceinline__ void prefetch_l2(const void *gmem)
     asm volatile("prefetch.global.L2 [%0];\n" ::"l"(gmem));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 // wait until at most n (0..3) of this thread's committed groups are pending
 __device__ __forceinline__ void cp_async_wait_pending(int n)
 {
@@ -242,10 +241,11 @@ __device__ __forceinline__ void pose_frame(const RotRec &rr, const PoseRec &pr, 
         c[a] = (fmaf(Rf[0 * 3 + a], pr.tf[0], fmaf(Rf[1 * 3 + a], pr.tf[1], Rf[2 * 3 + a] * pr.tf[2])) - rr.of[a]) * ih;
 }
 
-// One lattice row (jy, jz) of one pose: set the bits of the voxels inside the
-// probe.  The FP32 interval from the radial quadratic and the axial slab is
-// only a starting point: the exact end voxels are found by classifying
-// neighbours (an interval, since the cylinder is convex), with the exact
+// One lattice row (jy, jz) of one pose whose axis lies nearly along the row: set
+// the bits of the voxels inside the probe.  The radial ends of such a row are ill
+// conditioned: the FP32 interval only drops rows and gives the last voxel to
+// start from; the ends are found by classifying voxels from the row's start and
+// around that one (an interval, since the cylinder is convex), with the exact
 // FP64 predicate deciding inside the FP32 error band.
 template <int N>
 __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, int jz, float rv2, float lv, float mr,
@@ -258,7 +258,6 @@ __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, 
     float l0[3];
     for (int k = 0; k < 3; ++k) l0[k] = fmaf(B[0 * 3 + k], dxv, fmaf(B[1 * 3 + k], dyv, B[2 * 3 + k] * dzv));
     float lo = -1e30f, hi = 1e30f;
-    int wide = 2;
     if (Aq > 1e-6f) {
         float Bq = fmaf(l0[0], bx[0], l0[1] * bx[1]);
         float Cq = fmaf(l0[0], l0[0], l0[1] * l0[1]) - rv2;
@@ -267,11 +266,9 @@ __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, 
         float sq = sqrtf(fmaxf(disc, 0.f));
         lo = (-Bq - sq) / Aq;
         hi = (-Bq + sq) / Aq;
-        if (Aq < 0.05f) wide = N;
     } else {
         float Cq = fmaf(l0[0], l0[0], l0[1] * l0[1]) - rv2;
         if (Cq > mr + 1e-2f) return;
-        wide = N;
     }
     if (fabsf(bx[2]) >= 1e-3f) {
         float za = -l0[2] / bx[2], zb = (lv - l0[2]) / bx[2];
@@ -284,19 +281,10 @@ __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, 
         if (fmaxf(zA, zB) < -0.3f || fminf(zA, zB) > lv + 0.3f) return;
     }
     if (lo > hi + 2.f) return;
-    lo = fmaxf(lo, -4.f);
-    hi = fminf(hi, (float)N + 4.f);
-    const int jmax = min(N - 1, (int)ceilf(hi) + wide);
-    int jl = min(N - 1, max(0, (int)ceilf(lo)));
-    if (wide > 2) jl = max(0, (int)floorf(lo) - wide);
-    if (jl > jmax) return;
-    if (classify(l0, bx, jl, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz)) {
-        while (jl > 0 && classify(l0, bx, jl - 1, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz)) --jl;
-    } else {
-        do { ++jl; } while (jl <= jmax && !classify(l0, bx, jl, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz));
-        if (jl > jmax) return;
-    }
-    int jr = max(jl, min(N - 1, (int)floorf(hi)));
+    int jl = 0;
+    while (jl < N && !classify(l0, bx, jl, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz)) ++jl;
+    if (jl == N) return;
+    int jr = max(jl, (int)floorf(fminf(hi, (float)(N - 1))));
     if (classify(l0, bx, jr, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz)) {
         while (jr < N - 1 && classify(l0, bx, jr + 1, rv2, lv, mr, mz, rr, pr, h, r2d, Ld, jy, jz)) ++jr;
     } else {
@@ -321,9 +309,9 @@ __device__ __forceinline__ void vox_row(const float *B, const float *c, int jy, 
 // ends of the union can have any.  Lanes whose axis is nearly along the row
 // classify their row voxel by voxel with vox_row.
 //
-// Bound by instruction issue: at N = 128 and 5000 poses a rotation walked 144 000
-// rows of 270 warp instructions when every lane settled its own two ends (44.0 us
-// a rotation, now 18.3; 6.2 -> 3.5 us at N = 64 and 2000 poses).
+// Bound by instruction issue (72 % of the slots at N = 128): 144 000 rows a
+// rotation of 5000 poses, 18.3 us; 3.5 us at N = 64 and 2000 poses.  Every lane
+// settling its own two ends takes 270 warp instructions a row (44.0 and 6.2 us).
 template <int N>
 __device__ void voxelise_slab(const Geo &g, const RotRec &rr, const PoseRec *poses, int P, int jz, uint32_t *bits,
                               int *next_chunk)
@@ -934,10 +922,11 @@ cudaError_t launch_rot_export(const Geo &g, const ReqDev *reqs, const RotRec *ro
 // non-contact poses skip the addition and keep the plain result bit for bit.
 // Bound by the memory traffic of Y and Z and the chain of its exchanges: the
 // inputs come straight from global memory into registers, the next tile's on
-// their way during the current one, and blocks of 16 columns (64 to 256 threads)
-// leave four to eight of them on an SM.  With 32 columns staged by 8-byte
-// cp.async and the second spectrum read again per rotation, a rotation took 0.58,
-// 3.74 us (plain, N = 32, 64) and 30.3 us (DUAL, N = 96); now 0.33, 2.55 and 19.2.
+// their way during the current one, and blocks of 16 columns are small enough for
+// several on an SM (ZpassCfg::MINB: 8 at canvas 64, 6 at 128 and 3 at 192, with
+// DUAL 8, 4 and 2; other numbers with the alternative radix plans).  0.33 and 2.55 us a rotation at N = 32 and 64, 19.2 at N = 96 with
+// labels; with 32 columns staged by 8-byte cp.async and the second spectrum read
+// again for every rotation 0.58, 3.74 and 30.3.
 // ---------------------------------------------------------------------------
 template <int M, bool DUAL, int V = 0> struct ZpassCfg {
     static constexpr int COLS = M == 256 ? 32 : 16, NT = Plan<M, V>::T * COLS;
@@ -1114,10 +1103,10 @@ cudaError_t launch_zpass(const Geo &g, int B, int group, const float2 *Y, const 
 // The plane lives in the CTA's registers: a thread holds RA columns' share in
 // phase 1 and RB rows' share in phase 2, and the stages exchange in place through
 // one [M][H + 1] buffer (odd pitch: a warp's 32 rows of one column and its 32
-// columns of one row both hit distinct banks).  Five to nine block barriers a
-// plane (two per exchange), where rounds of 32 columns and rows through a second
-// buffer took about 24 with half as many warps on an SM: 0.53, 4.35, 21.2 us a
-// rotation at N = 32, 64, 96; now 0.40, 3.29, 16.9.
+// columns of one row both hit distinct banks).  Bound by the chain of its five to
+// nine block barriers a plane (two per exchange): 0.40, 3.29, 16.9 us a rotation at
+// N = 32, 64, 96; rounds of 32 columns and rows through a second buffer take about
+// 24 barriers with half as many warps on an SM (0.53, 4.35, 21.2 us).
 // ---------------------------------------------------------------------------
 template <int M, int V = 0> struct PlaneRegCfg {
     static constexpr int H = M / 2, VH = HasPlan<H, V>::value ? V : 0, PP = H + 1;
