@@ -269,11 +269,11 @@ def serving_experiment(ctx, synth):
 # 8-rotation launch of `bench.py --ncu-case` (dram__bytes_read.sum + dram__bytes_write.sum); a launch of B rotations is scaled from them by B/8
 # (the z pass's spectrum reads apart: zpass_spectrum_reads).  A kernel changed since its capture has no entry.
 # That z pass launch has three blocks per block column, each reading its part of the spectrum once.  The
-# voxeliser's smsp__inst_executed.sum is over a search of 256 SF rotations of the same workload (20 to 39 M
+# voxeliser's smsp__inst_executed.sum is over a search of 256 SF rotations of the same workload (20 to 37 M
 # a rotation).
 NCU_DRAM_BYTES_PER_ROT = {"plane": (545357312 + 3463168) / 8, "fwd2d": (18613248 + 229198848) / 8,
-                          "zpass": (476177920 - 3 * 68157440 + 485797888) / 8, "voxelise": (908288 + 0) / 8}
-NCU_WARP_INST_PER_ROT = {"voxelise": 6580964989 / 256}
+                          "zpass": (476177920 - 3 * 68157440 + 485797888) / 8, "voxelise": (907264 + 0) / 8}
+NCU_WARP_INST_PER_ROT = {"voxelise": 6458504365 / 256}
 # SMs x warp schedulers: one warp instruction issued per scheduler per clock
 ISSUE_SLOTS = 152 * 4
 
